@@ -128,7 +128,8 @@ struct sphfsi_ctx {
     Batch bt{};
     Inst *d_inst = nullptr;
     Ctl *ctl = nullptr;
-    std::vector<std::pair<void *, size_t>> allocs;   // every device allocation (pointer, bytes)
+    std::vector<std::pair<void *, size_t>> allocs;   // every device allocation of the state (pointer, bytes)
+    std::vector<void *> scratch;                     // device allocations that are no part of a checkpoint
     // graph replay
     cudaGraphExec_t gexec = nullptr;
     double graph_dt = 0.0;
@@ -177,6 +178,18 @@ int dalloc(sphfsi_ctx *c, T **p, size_t count)
     cudaMemsetAsync(q, 0, sizeof(T) * count, c->st);
     c->allocs.push_back({q, sizeof(T) * count});
     *p = (T *)q;
+    return SPHFSI_OK;
+}
+
+// the same for memory that no checkpoint holds: plans derived from the set-up
+// and buffers that carry nothing from one step to the next
+template <typename T>
+int dscratch(sphfsi_ctx *c, T **p, size_t count)
+{
+    const int rc = dalloc(c, p, count);
+    if (rc) return rc;
+    c->scratch.push_back(c->allocs.back().first);
+    c->allocs.pop_back();
     return SPHFSI_OK;
 }
 
@@ -520,6 +533,54 @@ int body_neighbours(sphfsi_ctx *c, std::vector<int> &ptr, std::vector<int> &idx)
             for (int len : clen[ch]) ptr.push_back(ptr.back() + len);
         }
     }
+    return SPHFSI_OK;
+}
+
+// Plan of the windowed sub-step kernel (one body): CTA c owns the particles
+// [c own, (c + 1) own), its window runs from the smallest to the largest
+// particle that they and their neighbours are, and it exchanges particles
+// with the CTAs whose particles its window reaches and those whose windows
+// reach its own particles.  Rows of nbi are ascending, so a row's ends bound it.
+int solid_windows(sphfsi_ctx *c, const std::vector<int> &ptr, const std::vector<int> &nbi)
+{
+    Solid &S = c->S;
+    S.win_ctas = 0;
+    if (c->B != 1 || S.n == 0) return SPHFSI_OK;
+    int dev = 0, nsm = 0, own = 0, threads = 0;
+    TRY(cuda_rc(cudaGetDevice(&dev)));
+    TRY(cuda_rc(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)));
+    solid_window_shape(c->dim, S.n, nsm, &own, &threads);
+    const int ctas = (S.n + own - 1) / own;
+    std::vector<int4> win(ctas);
+    std::vector<int2> wait(ctas);
+    int slots = 0;
+    for (int k = 0; k < ctas; k++) {
+        const int a0 = k * own, a1 = std::min(a0 + own, S.n);
+        int lo = a0, hi = a1;
+        for (int a = a0; a < a1; a++)
+            if (ptr[a + 1] > ptr[a]) {
+                lo = std::min(lo, nbi[ptr[a]]);
+                hi = std::max(hi, nbi[ptr[a + 1] - 1] + 1);
+            }
+        win[k] = make_int4(a0, a1 - a0, lo, hi - lo);
+        wait[k] = make_int2(lo / own, (hi - 1) / own);
+        slots = std::max(slots, hi - lo);
+    }
+    for (int k = 0; k < ctas; k++)   // both directions
+        for (int j = win[k].z / own; j <= (win[k].z + win[k].w - 1) / own; j++) {
+            wait[j].x = std::min(wait[j].x, k);
+            wait[j].y = std::max(wait[j].y, k);
+        }
+    if (!solid_window_fits(c->dim, ctas, threads, slots, own)) return SPHFSI_OK;
+    TRY(dscratch(c, &S.win, ctas));
+    TRY(dscratch(c, &S.win_wait, ctas));
+    TRY(dscratch(c, &S.win_flag, 32 * (size_t)ctas));
+    TRY(upload(c, S.win, win));
+    TRY(upload(c, S.win_wait, wait));
+    S.win_ctas = ctas;
+    S.win_threads = threads;
+    S.win_slots = slots;
+    S.win_own = own;
     return SPHFSI_OK;
 }
 
@@ -1155,6 +1216,7 @@ int sphfsi_finalize(sphfsi_ctx *c)
         TRY(dalloc(c, &S.nb, S.nnz));
         TRY(launch_solid_setup_fill(c->bt, S, d_nbi, D, c->st));
         if (D == 2) TRY(halo_maps(c, ptr, nbi));
+        TRY(solid_windows(c, ptr, nbi));
     }
     TRY(cuda_rc(cudaStreamSynchronize(c->st)));
     for (int k = 0; k < sphfsi_ctx::kEvents; k++) TRY(cuda_rc(cudaEventCreate(&c->ev[k])));
@@ -1693,6 +1755,9 @@ int sphfsi_set_state(sphfsi_ctx *c, const void *blob, int64_t bytes)
         TRY(cuda_rc(cudaMemcpy(a.first, p, a.second, cudaMemcpyHostToDevice)));
         p += a.second;
     }
+    // after a time-out the CTAs of the windowed kernel may have published
+    // different numbers of phases
+    if (c->S.win_ctas) TRY(cuda_rc(cudaMemset(c->S.win_flag, 0, sizeof(unsigned) * 32 * (size_t)c->S.win_ctas)));
     // steps are allowed again unless the checkpoint itself was taken after a
     // scan that gave up or a step that ran away
     int fail = 0;
@@ -2194,6 +2259,7 @@ void sphfsi_destroy(sphfsi_ctx *c)
     if (c->join_ev) cudaEventDestroy(c->join_ev);
     if (c->side) cudaStreamDestroy(c->side);
     for (auto &a : c->allocs) cudaFree(a.first);
+    for (void *p : c->scratch) cudaFree(p);
     delete c;
 }
 

@@ -262,6 +262,15 @@ struct Solid {
     int *key, *perm, *cstart, *ccount, *cell_of;
     int *sperm;                  // sorted slot -> particle (large batches: ranks, then records)
     unsigned *bar;            // grid barrier: [0] arrivals, [1] generation
+    // windowed sub-step kernel (single bodies): CTA c owns consecutive
+    // particles and reads those of one window of the body around them
+    int4 *win;                // per CTA: (first particle, particles, first of the window, window's particles)
+    int2 *win_wait;           // per CTA: first and last CTA that it exchanges particles with
+    unsigned *win_flag;       // per CTA, 128 bytes apart: phases published so far (never reset by a step)
+    int win_ctas;             // 0: no window plan (a batch, no body, or a window beyond the shared memory)
+    int win_threads;          // threads per CTA
+    int win_slots;            // largest window
+    int win_own;              // most particles of a CTA
     unsigned *queue;          // persistent solid kernel: next instance to take
     int force_grid_path;      // 1: always use the cooperative-grid sub-step kernel
     int force_lane_path;      // 2-D cluster kernel: 0 one thread per particle, 1 four lanes, 2 two threads
@@ -472,6 +481,10 @@ int launch_debug_pairs(const Batch &bt, const Fluid &f, const Walls &w, const So
 int launch_solid_setup_fill(const Batch &bt, Solid &s, const int *nbi, int dim, cudaStream_t st);
 // P0: host copy of instance 0's constants (used when the batch holds one instance)
 int launch_solid_substeps(const Batch &bt, Solid &s, const Phys &P0, int dim, int *path, cudaStream_t st);
+// plan of the windowed sub-step kernel: particles and threads per CTA, and
+// whether the device can hold the grid with these windows (sph_solid.cu)
+void solid_window_shape(int dim, int n, int nsm, int *own, int *threads);
+int solid_window_fits(int dim, int ctas, int threads, int slots, int own);
 // learned sub-stepper: features into x (n x 64), then, from the network's
 // outputs (n x 16), candidate, residual and accept / reject (sph_solid.cu)
 int launch_learn_features(const Batch &bt, const Solid &s, float *x, int dim, cudaStream_t st);

@@ -1478,10 +1478,430 @@ static int launch_solid_cluster(const Batch &bt, Solid &s, const Phys &P0, int d
     return launch_persistent(k_solid_cluster<3>, kCThreads, ctas, bt, s, mcl[3], st);
 }
 
+// ---------------------------------------------------------------------------
+// Windowed variant for one body of any size whose windows fit shared memory:
+// a cooperative grid of at most one CTA per SM.  CTA c owns up to a few
+// hundred consecutive particles (device locality order) and keeps the stress
+// Q = P B0 and the velocity of a window of consecutive particles around them,
+// wide enough to hold every neighbour, in shared memory.
+//
+// What bounds the plain grid kernel above is latency: one thread walks a
+// particle's 20 to 80 neighbours with two dependent L2 loads each, and every
+// phase ends in a barrier of all blocks on one counter.  Here:
+//  - L lanes share a particle's list (8 in 3-D, 4 in 2-D: a group reads whole
+//    128- or 64-byte lines of it, kWinU entries in flight per lane) and read
+//    the neighbours' Q or v from shared memory; each window particle crosses
+//    L2 once per CTA and phase instead of once per pair;
+//  - thread t < n keeps the state of particle t (H, B0, FP64 position and
+//    sums) in registers for all K sub-steps, so the stress runs with every
+//    lane busy;
+//  - a CTA waits only for the CTAs it exchanges particles with: each counts
+//    the phases it has published in its own flag, and waits until theirs have
+//    got as far.  A CTA's wait set holds every CTA whose window reaches its
+//    particles and every CTA its window reaches, so a CTA that has passed the
+//    wait of a phase also knows that nobody still reads what it writes next:
+//    Q of sub-step k is read before v of sub-step k is published.
+// Flags count on from launch to launch (every CTA publishes the same number
+// of phases), so no launch has to clear them.
+// Waits are bounded: on a time-out the status bit is set and the CTA returns;
+// its neighbours then time out as well.
+// Measured (GB300, the sub-steps of one coarse step, stage events): 2-D gate
+// of 6400 particles, 25 sub-steps, 494 us with the plain grid kernel, 122 us
+// here; 3-D plates of 8160 and 64 640 particles, 14 sub-steps, 665 and 1732 us
+// against 120 and 505 us (beside the fluid loops); entries held in registers
+// instead of read in every phase: 166 -> 122, 140 -> 120 us; 3-D plate of
+// 1408 particles, 10 sub-steps, 275 us with the cluster kernel, 80 us here.
+// ---------------------------------------------------------------------------
+constexpr int kWinThreads = 512;
+// list entries a lane holds or keeps in flight: with the lanes per particle
+// (4 in 2-D, 8 in 3-D) 20 and 80 entries, the lattice's neighbour counts
+template <int D> constexpr int kWinL = D == 3 ? 8 : 4;
+template <int D> constexpr int kWinU = D == 3 ? 10 : 5;
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(unsigned *p, unsigned v)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// HELD: every group has one particle and its lanes hold all of its entries in
+// registers for the whole step; otherwise a group walks several particles (or
+// longer lists) and streams their entries from L2 in every phase.
+template <int D, bool HELD>
+__global__ void __launch_bounds__(kWinThreads, 1) k_solid_window(Batch bt, Solid s)
+{
+    if (step_failed(bt)) return;   // uniform over the grid
+    const Phys &P = bt.I[0].P;
+    Ctl *ctl = bt.ctl;
+    if (ctl->learned_ok) return;   // the learned step was accepted: no sub-steps
+    constexpr int DD = D * D, QR = D == 3 ? 3 : 1, L = kWinL<D>, U = HELD ? kWinU<D> : 5;
+    extern __shared__ float4 s_win[];
+    const int4 win = s.win[blockIdx.x];
+    const int2 ww = s.win_wait[blockIdx.x];
+    const int a0 = win.x, n = win.y, lo = win.z, nw = win.w;
+    float4 *const sQ = s_win;                       // [QR][win_slots]
+    float4 *const sV = s_win + QR * s.win_slots;    // [win_slots]
+    float *const sM = (float *)(sV + s.win_slots);  // [n][DD]: sums of the pair loops
+    const int t = threadIdx.x, T = blockDim.x, lane = t % L, g = t / L, G = T / L;
+    const int K = ctl->K;
+    const double dt = ctl->dt, dtsd = ctl->dts, hdtsd = 0.5 * dtsd;
+    const float dts = (float)dtsd, hdts = 0.5f * dts;
+    const float inv_rhoS = 1.0f / P.rhoS, inv_mS = 1.0f / P.mS;
+    unsigned *const my_flag = s.win_flag + 32 * blockIdx.x;
+    unsigned ep = *my_flag;   // this CTA's own count: no other CTA writes it
+
+    // phase end: this CTA's particles are in global memory
+    auto publish = [&]() {
+        ep++;
+        __syncthreads();
+        if (t == 0) st_release(my_flag, ep);   // cumulative over the CTA's writes (barrier above)
+    };
+    // wait until the CTAs of the wait set have published as many phases
+    auto wait = [&]() {
+        bool ok = true;
+        if (t < 32) {
+            for (int c = ww.x + t; c <= ww.y; c += 32) {
+                long long it = 0;
+                while ((int)(ld_acquire(s.win_flag + 32 * c) - ep) < 0) {
+                    if (++it > bt.spin) {
+                        ok = false;
+                        break;
+                    }
+                }
+            }
+        }
+        ok = __syncthreads_and(ok);
+        if (!ok && t == 0) atomicOr(&ctl->status, ST_TIMEOUT);
+        return ok;
+    };
+    // the window's particles of the other CTAs
+    auto load_v = [&]() {
+        for (int k = t; k < nw; k += T)
+            if ((unsigned)(lo + k - a0) >= (unsigned)n) sV[k] = __ldcg(&s.v4[lo + k]);
+        __syncthreads();
+    };
+    auto load_Q = [&]() {
+        for (int k = t; k < nw * QR; k += T) {
+            const int j = k / QR, r = k - j * QR;
+            if ((unsigned)(lo + j - a0) >= (unsigned)n) sQ[r * s.win_slots + j] = __ldcg(&s.Q4[(size_t)QR * lo + k]);
+        }
+        __syncthreads();
+    };
+    // pair loops: sums of particle p of the CTA into sM[p]; a lane takes every
+    // L-th entry, U at a time (no entry: a zero gradient on the particle itself)
+    float4 e[U];
+    auto load_entries = [&](int q, int q1, int ia) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            e[u] = make_float4(0.f, 0.f, 0.f, __int_as_float(ia));
+            if (q + u * L < q1) {
+                e[u] = __ldg(&s.nb[q + u * L]);
+                e[u].w = __int_as_float(__float_as_int(e[u].w) - lo);
+            }
+        }
+    };
+    if (HELD) {
+        const int p = g < n ? a0 + g : a0;
+        const int q0 = s.nb_ptr[p], q1 = g < n ? s.nb_ptr[p + 1] : q0;
+        load_entries(q0 + lane, q1, p - lo);
+    }
+    auto entries = [&](auto &&begin, auto &&pair, auto &&end) {
+        if (HELD) {
+            begin((g < n ? a0 + g : a0) - lo);
+#pragma unroll
+            for (int u = 0; u < U; u++) pair(e[u], __float_as_int(e[u].w));
+            end(g < n, g);
+        } else {
+            for (int p0 = 0; p0 < n; p0 += G) {
+                const int p = p0 + g;
+                const bool act = p < n;
+                const int a = a0 + (act ? p : 0);
+                const int q0 = s.nb_ptr[a], q1 = act ? s.nb_ptr[a + 1] : q0;
+                begin(a - lo);
+                for (int q = q0 + lane; q < q1; q += L * U) {
+                    load_entries(q, q1, a - lo);
+#pragma unroll
+                    for (int u = 0; u < U; u++) pair(e[u], __float_as_int(e[u].w));
+                }
+                end(act, p);
+            }
+        }
+        __syncthreads();
+    };
+    auto reduce = [&](float v) {
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    // [sum_b (v_b - v_a) (x) V0 grad0 W_ab]
+    auto rate_sums = [&]() {
+        float4 va;
+        float M[DD];
+        entries(
+            [&](int ia) {
+                va = sV[ia];
+#pragma unroll
+                for (int i = 0; i < DD; i++) M[i] = 0.0f;
+            },
+            [&](const float4 &e, int ib) {
+                const float4 vb = sV[ib];
+                const float dv[3] = {vb.x - va.x, vb.y - va.y, vb.z - va.z}, ge[3] = {e.x, e.y, e.z};
+#pragma unroll
+                for (int i = 0; i < D; i++)
+#pragma unroll
+                    for (int j = 0; j < D; j++) M[i * D + j] += dv[i] * ge[j];
+            },
+            [&](bool act, int p) {
+#pragma unroll
+                for (int i = 0; i < DD; i++) M[i] = reduce(M[i]);
+                if (act && lane == 0)
+#pragma unroll
+                    for (int i = 0; i < DD; i++) sM[p * DD + i] = M[i];
+            });
+    };
+    // sum_b (Q_a + Q_b) V0 grad0 W_ab
+    auto force_sums = [&]() {
+        float4 qa[QR];
+        float f[3];
+        entries(
+            [&](int ia) {
+#pragma unroll
+                for (int r = 0; r < QR; r++) qa[r] = sQ[r * s.win_slots + ia];
+                f[0] = f[1] = f[2] = 0.0f;
+            },
+            [&](const float4 &e, int ib) {
+                if (D == 2) {
+                    const float4 qb = sQ[ib];
+                    f[0] += (qa[0].x + qb.x) * e.x + (qa[0].y + qb.y) * e.y;
+                    f[1] += (qa[0].z + qb.z) * e.x + (qa[0].w + qb.w) * e.y;
+                } else {
+#pragma unroll
+                    for (int r = 0; r < QR; r++) {
+                        const float4 qb = sQ[r * s.win_slots + ib];
+                        f[r] += (qa[r].x + qb.x) * e.x + (qa[r].y + qb.y) * e.y + (qa[r].z + qb.z) * e.z;
+                    }
+                }
+            },
+            [&](bool act, int p) {
+#pragma unroll
+                for (int k = 0; k < D; k++) f[k] = reduce(f[k]);
+                if (act && lane == 0)
+#pragma unroll
+                    for (int k = 0; k < D; k++) sM[p * DD + k] = f[k];
+            });
+    };
+
+    // state of particle t
+    const bool own = t < n;
+    const int a = a0 + (own ? t : 0), slot = a - lo;
+    // (Hr, vr: what the FP32 sums H and v have rounded off so far this step,
+    // carried into the next addition, so that a step rounds its state once
+    // instead of at every sub-step)
+    float H[DD], B[DD], fF[3] = {0.f, 0.f, 0.f}, vmax = 0.0f, amax = 0.0f;
+    float Hr[DD], vr[3] = {0.f, 0.f, 0.f};
+    double x = 0, y = 0, z = 0, xs = 0, ys = 0, zs = 0, as[3] = {0, 0, 0};
+    bool cons = true;
+#pragma unroll
+    for (int i = 0; i < DD; i++) Hr[i] = 0.0f;
+    auto add = [](float &sum, float &rest, float d) {
+        const float y = __fadd_rn(d, rest), t = __fadd_rn(sum, y);
+        rest = __fsub_rn(y, __fsub_rn(t, sum));
+        sum = t;
+    };
+    if (own) {
+#pragma unroll
+        for (int i = 0; i < DD; i++) {
+            H[i] = s.H[9 * a + i];
+            B[i] = s.B0[9 * a + i];
+        }
+        for (int k = 0; k < D; k++) fF[k] = s.fF[3 * a + k];
+        x = xs = s.x[a];
+        y = ys = s.y[a];
+        if (D == 3) z = zs = s.z[a];
+        cons = s.cons[a] != 0;
+    }
+    for (int k = t; k < nw; k += T) sV[k] = __ldcg(&s.v4[lo + k]);
+    __syncthreads();
+
+    // half drifts of H and the position with dH/dt = M B0, then the stress of
+    // the next sub-step
+    auto drift = [&](bool second, bool first) {
+        rate_sums();
+        if (own) {
+            const float *M = sM + t * DD;
+#pragma unroll
+            for (int i = 0; i < D; i++)
+#pragma unroll
+                for (int j = 0; j < D; j++) {
+                    float hd = 0.0f;
+#pragma unroll
+                    for (int k = 0; k < D; k++) hd += M[i * D + k] * B[k * D + j];
+                    if (second) add(H[i * D + j], Hr[i * D + j], hdts * hd);
+                    if (first) add(H[i * D + j], Hr[i * D + j], hdts * hd);
+                }
+            if (!cons) {
+                const float4 v = sV[slot];
+                const int reps = (second ? 1 : 0) + (first ? 1 : 0);
+                for (int r = 0; r < reps; r++) {
+                    x = x + hdtsd * (double)v.x;
+                    y = y + hdtsd * (double)v.y;
+                    if (D == 3) z = z + hdtsd * (double)v.z;
+                }
+            }
+            if (first) {
+                float Q[9];
+                stress_QB<D>(H, B, P.mu, P.lam, Q);
+                if (D == 2) {
+                    const float4 q = make_float4(Q[0], Q[1], Q[2], Q[3]);
+                    sQ[slot] = q;
+                    __stcg(&s.Q4[a], q);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < QR; r++) {
+                        const float4 q = make_float4(Q[3 * r], Q[3 * r + 1], Q[3 * r + 2], 0.0f);
+                        sQ[r * s.win_slots + slot] = q;
+                        __stcg(&s.Q4[(size_t)QR * a + r], q);
+                    }
+                }
+            }
+        }
+        if (first) publish();
+    };
+
+    drift(false, true);   // start of step: dH/dt(v^0), first half drift of sub-step 0, stress
+    for (int kk = 0; kk < K; kk++) {
+        // (B) force loop and kick
+        if (!wait()) return;
+        load_Q();
+        force_sums();
+        if (own && !cons) {
+            float av[3] = {0.f, 0.f, 0.f}, a2 = 0.0f;
+            float4 v = sV[slot];
+#pragma unroll
+            for (int k = 0; k < D; k++) {
+                av[k] = sM[t * DD + k] * inv_rhoS + fF[k] * inv_mS + P.g[k];
+                as[k] += dtsd * (double)av[k];
+                a2 += av[k] * av[k];
+            }
+            add(v.x, vr[0], dts * av[0]);
+            add(v.y, vr[1], dts * av[1]);
+            if (D == 3) add(v.z, vr[2], dts * av[2]);
+            sV[slot] = v;
+            __stcg(&s.v4[a], v);
+            amax = max_keep_nan(amax, a2);
+            vmax = max_keep_nan(vmax, v.x * v.x + v.y * v.y + v.z * v.z);
+        }
+        publish();
+        // (C) deformation rate at v^{k+1}, second half drift; next first half and stress
+        if (!wait()) return;
+        load_v();
+        drift(true, kk + 1 < K);
+    }
+    // write back; a8 time averages (reading R14)
+    if (own) {
+#pragma unroll
+        for (int i = 0; i < DD; i++) s.H[9 * a + i] = H[i];
+        s.x[a] = x;
+        s.y[a] = y;
+        if (D == 3) s.z[a] = z;
+        const double idt = 1.0 / dt;
+        s.vbar[3 * a] = (x - xs) * idt;
+        s.vbar[3 * a + 1] = (y - ys) * idt;
+        s.vbar[3 * a + 2] = D == 3 ? (z - zs) * idt : 0.0;
+        for (int k = 0; k < 3; k++) s.abar[3 * a + k] = as[k] * idt;
+    }
+    float vm = warp_max(vmax), am = warp_max(amax);
+    if ((t & 31) == 0) {
+        atomic_max_pos(&ctl->vmaxS, sqrtf(vm));
+        atomic_max_pos(&ctl->amaxS, sqrtf(am));
+    }
+}
+
+static size_t window_smem(int dim, int slots, int own)
+{
+    return (size_t)slots * 16 * (dim == 3 ? 4 : 2) + (size_t)own * dim * dim * sizeof(float);
+}
+
+// Shape of the windowed kernel for a body of n particles: particles per CTA
+// and threads per CTA.  One CTA per SM at most; a small body is spread over
+// fewer CTAs of kWinMinOwn particles, since a CTA's phase costs a few L2
+// round trips however little it holds.
+void solid_window_shape(int dim, int n, int nsm, int *own, int *threads)
+{
+    const int L = dim == 3 ? kWinL<3> : kWinL<2>, least = 32;
+    int P = (n + nsm - 1) / nsm;
+    if (P < least) P = least;
+    int T = (P * L + 31) / 32 * 32;
+    if (T > kWinThreads) T = kWinThreads;
+    if (T < (P + 31) / 32 * 32) T = (P + 31) / 32 * 32;
+    *own = P;
+    *threads = T;
+}
+
+// Can the device hold the plan's grid at once?  (0: no)
+int solid_window_fits(int dim, int ctas, int threads, int slots, int own)
+{
+    if (threads > kWinThreads || own > threads) return 0;
+    const size_t smem = window_smem(dim, slots, own);
+    int dev = 0, nsm = 0, most = 0, per = 0, least = 1 << 30;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (smem > (size_t)most) return 0;
+    auto query = [&](auto kern) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem) != cudaSuccess)
+            return false;
+        least = per < least ? per : least;
+        return true;
+    };
+    const bool ok = dim == 3 ? query(k_solid_window<3, true>) && query(k_solid_window<3, false>)
+                             : query(k_solid_window<2, true>) && query(k_solid_window<2, false>);
+    if (!ok) {
+        cudaGetLastError();
+        return 0;
+    }
+    return ctas <= least * nsm ? 1 : 0;
+}
+
+static int launch_solid_window(const Batch &bt, const Solid &s, int dim, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(s.win_ctas);
+    cfg.blockDim = dim3(s.win_threads);
+    cfg.dynamicSmemBytes = window_smem(dim, s.win_slots, s.win_own);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;   // all CTAs resident: they wait for one another
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const int L = dim == 3 ? kWinL<3> : kWinL<2>, U = dim == 3 ? kWinU<3> : kWinU<2>;
+    const bool held = s.win_own * L <= s.win_threads && s.max_nb <= L * U;
+    cudaError_t e;
+    if (dim == 2)
+        e = held ? cudaLaunchKernelEx(&cfg, k_solid_window<2, true>, bt, s)
+                 : cudaLaunchKernelEx(&cfg, k_solid_window<2, false>, bt, s);
+    else
+        e = held ? cudaLaunchKernelEx(&cfg, k_solid_window<3, true>, bt, s)
+                 : cudaLaunchKernelEx(&cfg, k_solid_window<3, false>, bt, s);
+    return e == cudaSuccess ? 0 : -3;
+}
+
+// 3-D bodies above this size take the windowed kernel instead of the cluster
+// kernel, whose lanes read every neighbour's three Q rows across the cluster
+constexpr int kWin3dFrom = 2048;
+
 int launch_solid_substeps(const Batch &bt, Solid &s, const Phys &P0, int dim, int *path, cudaStream_t st)
 {
     if (s.n == 0) return 0;
-    if (!s.force_grid_path) {
+    const bool window = s.win_ctas > 0 && bt.B == 1;
+    if (!s.force_grid_path && !(window && dim == 3 && s.n > kWin3dFrom && !s.force_lane_path)) {
         int cp = 1;
         int rc = launch_solid_cluster(bt, s, P0, dim, st, &cp);
         if (rc <= 0) {
@@ -1489,8 +1909,12 @@ int launch_solid_substeps(const Batch &bt, Solid &s, const Phys &P0, int dim, in
             return rc;
         }
     }
-    // cooperative grid kernel: one large body (a batch needs the cluster path)
+    // cooperative grid kernels: one large body (a batch needs the cluster path)
     if (bt.B != 1) return -7;
+    if (window) {
+        if (path) *path = 2;
+        return launch_solid_window(bt, s, dim, st);
+    }
     static int max_blocks[2] = {0, 0};
     int di = dim == 2 ? 0 : 1;
     if (max_blocks[di] == 0) {
