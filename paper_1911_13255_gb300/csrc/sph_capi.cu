@@ -991,6 +991,9 @@ int sphfsi_finalize(sphfsi_ctx *c)
     F.list_cap = D == 2 ? 64 : 128;
     TRY(dalloc(c, &F.nbl, (size_t)nf * F.list_cap));
     TRY(dalloc(c, &F.nbc, nf));
+    for (int p = 0; p < 2; p++) TRY(dscratch(c, &F.part[p], nf));
+    TRY(dscratch(c, &F.part_n, 2));
+    TRY(dscratch(c, &F.B4, nf));
     // held pair configuration: off (rebuilt every step); the first step builds it
     F.held_n = 1;
     TRY(dalloc(c, &F.held, 3));

@@ -214,6 +214,12 @@ struct Fluid {
     int list_cap;
     uint32_t *nbl;
     uint32_t *nbc;
+    // targets that the row build lists apart: [kPartNear] those with solid
+    // particles in their neighbour cells and overflowed rows, [kPartWall]
+    // those with wall neighbours and no solid particles
+    int *part[2];
+    int *part_n;
+    float4 *B4;           // boundary part of a target's density rate: coefficient on v^{n+1}, constant
 };
 
 // nbc flags: solid particles in one of the target's neighbour cells (the pair
@@ -221,6 +227,8 @@ struct Fluid {
 // target takes the cell visit for everything)
 constexpr uint32_t kListSolid = 1u << 22, kListOver = 1u << 23;
 constexpr uint32_t kListCountMask = 0x7ffu;
+constexpr uint32_t kListWalls = kListCountMask << 11;   // nW != 0
+enum : int { kPartNear = 0, kPartWall = 1 };
 
 // Static walls, binned once.
 struct Walls {

@@ -27,24 +27,12 @@ __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, con
         Pi = f.P4[i];
         Wi = f.W4[i];
         const float vi[3] = {Wi.x, Wi.y, Wi.z};
-        const float drhoi = Wi.w, rhoi = P.rho0 + Wi.w, pi = Pi.w;
+        const float drhoi = Wi.w, rhoi = P.rho0 + Wi.w;
         int cx, cy, cz;
         cell_xyz(f.cell_of[i], In, cx, cy, cz);
         const float inv2c0 = 0.5f / P.c0;
-        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        auto wall_pair = [&](int a, float ox, float oy, float oz) {
-            float d[3];
-            float r2 = rel_d<D>(Pi, w.A4[a], ox, oy, oz, d);
-            if (r2 >= P.rc2F) return;
-            rate += fs_pair_drho<D>(d, r2, vi, rhoi, pi, z4, z4, w.N4[a], P.VW, P);
-        };
-        auto solid_pair = [&](int b, float ox, float oy, float oz) {
-            float d[3];
-            float r2 = rel_d<D>(Pi, s.A4[b], ox, oy, oz, d);
-            if (r2 >= P.rc2F) return;
-            rate += fs_pair_drho<D>(d, r2, vi, rhoi, pi, s.VB4[b], s.AB4[b], s.N4[b], P.VS, P);
-        };
-        fluid_pairs<D, L, CP, FORM>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, P.rc2F, list, stride, ts,
+        auto none = [](int, float, float, float) {};
+        fluid_pairs<D, L, CP, FORM, kFluidOnly, true>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, P.rc2F, list, stride, ts,
                                 [&](int j) { return f.W4[j]; },
                                 [&](int, const float4 &, const float4 &Wj, const float *d, float r2, float, float,
                                     float) {
@@ -59,10 +47,15 @@ __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, con
                 // (v_i - v~_ij).grad_i W = -dW (U_L - U*), U* = (U_L + U_R)/2 + (p_i - p_j) / (2 rho c0)
                 float diff = 0.5f * (UL - UR) - eos_dp(drhoi, Wj.w, P) * inv2c0 / rb;
                 rate += __fdividef(P.mF, rhoj) * (-dW) * diff;
-            }, wall_pair, solid_pair);
+            }, none, none);
     }
     rate = group_sum<L>(rate);
     if (!act || lane != 0) return;
+    // walls and solid: the momentum loop's sums (fs_pair_force)
+    if (FORM != 3 || (f.nbc[i] & (kListSolid | kListWalls | kListOver))) {
+        const float4 Bi = f.B4[i];
+        rate += Bi.x * Wi.x + Bi.y * Wi.y + (D == 3 ? Bi.z * Wi.z : 0.0f) + Bi.w;
+    }
     const float vi[3] = {Wi.x, Wi.y, Wi.z};
     const float rhoi = P.rho0 + Wi.w;
     float rhodot = 2.0f * rhoi * rate;
@@ -111,7 +104,7 @@ int launch_density(const Batch &bt, const Fluid &f, const Walls &w, const Solid 
 {
     if (f.n == 0) return 0;
     if (f.n >= kMaxPairTargets) return -7;
-    SPH_LAUNCH_PAIRS(k_density, f.n, bt, f, w, s);
+    SPH_LAUNCH_PAIRS(k_density, f.n, 0, bt, f, w, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -203,13 +196,13 @@ __device__ __forceinline__ ff W_ff_shape(const float4 &Pi, const float4 &Li, con
     return ff_mul(ff_sqr(a2), bq);
 }
 
-template <int D, int L, bool CP, int FORM>
+template <int D, int L, bool CP, int FORM, int SETS>
 __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int i,
                                                  bool act_, int lane, uint32_t *list, int stride, const TileSrc *ts)
 {
     const int b = act_ ? f.inst[i] : 0;
     // the L lanes of a particle share its instance, so this is group-uniform
-    const bool act = act_ && bt.ctl[b].reinit;
+    const bool act = act_ && bt.ctl[b].reinit && (SETS == kAllSets || !(f.nbc[i] & (kListSolid | kListOver)));
     const Inst &In = bt.I[b];
     const Grid &g = In.g;
     const Phys &P = In.P;
@@ -232,7 +225,7 @@ __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, cons
             sS = ff_add(sS, W_ff_shape<D>(Pi, Li, Aq, s.L4[q], ox, oy, oz, g, P));
         };
         // the screen passes pairs up to 1.0001 (2 h)^2; W_ff_shape returns 0 beyond the support
-        fluid_pairs<D, L, CP, FORM>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, screen, list, stride, ts,
+        fluid_pairs<D, L, CP, FORM, SETS, SETS == kAllSets>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, screen, list, stride, ts,
                                 [&](int j) { return f.L4[j]; },
                                 [&](int, const float4 &Pj, const float4 &Lj, const float *, float, float ox, float oy,
                                     float oz) {
@@ -252,22 +245,35 @@ __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, cons
     f.V4[i].w = drho;
 }
 
+// Row form: the targets near solid particles and those of overflowed rows take
+// a warp each, in the first blocks (as in k_momentum; the walls, whose pairs
+// cost no more than the fluid's here, stay with the rest).
 template <int D, int L, bool CP, bool TILE, int FORM>
-__global__ void __launch_bounds__(kMaxBlock) k_reinit(Batch bt, Fluid f, Walls w, Solid s)
+__global__ void __launch_bounds__(kMaxBlock, D == 2 && FORM != 1 ? 5 : (D == 3 && FORM == 1 ? 3 : 4)) k_reinit(Batch bt, Fluid f, Walls w, Solid s)
 {
     pdl_enter();
     if (step_failed(bt)) return;   // the step's cell starts are not valid
     extern __shared__ __align__(16) uint8_t s_dyn[];
     uint32_t *const list = (uint32_t *)s_dyn + threadIdx.x;
     const int stride = blockDim.x;
-    if constexpr (!TILE) {
+    if constexpr (FORM == 3) {
+        const int nn = part_blocks(f.n, kPartNear, blockDim.x), k = blockIdx.x;
+        if (k < nn) {
+            part_loop<32>(f, kPartNear, k, nn, [&](int i, bool act, int lane) {
+                reinit_one<D, 32, CP, FORM, kAllSets>(bt, f, w, s, i, act, lane, nullptr, 0, nullptr);
+            });
+        } else {
+            const int t = (k - nn) * blockDim.x + threadIdx.x;
+            reinit_one<D, L, CP, FORM, kFluidWall>(bt, f, w, s, t / L, t / L < f.n, t % L, nullptr, 0, nullptr);
+        }
+    } else if constexpr (!TILE) {
         const int t = blockIdx.x * blockDim.x + threadIdx.x;
-        reinit_one<D, L, CP, FORM>(bt, f, w, s, t / L, t / L < f.n, t % L, list, stride, nullptr);
+        reinit_one<D, L, CP, FORM, kAllSets>(bt, f, w, s, t / L, t / L < f.n, t % L, list, stride, nullptr);
     } else {
         if (!bt.ctl[f.tiles[blockIdx.x].x].reinit) return;   // not a reinitialisation step of this instance
         tile_loop<D, L>(bt, f, f.L4, s_dyn + (CP ? (size_t)kListBytes * blockDim.x : 0),
                         [&](int i, bool act, const TileSrc *ts) {
-                            reinit_one<D, L, CP, FORM>(bt, f, w, s, i, act, (int)threadIdx.x % L, list, stride, ts);
+                            reinit_one<D, L, CP, FORM, kAllSets>(bt, f, w, s, i, act, (int)threadIdx.x % L, list, stride, ts);
                         });
     }
 }
@@ -276,7 +282,7 @@ int launch_reinit(const Batch &bt, const Fluid &f, const Walls &w, const Solid &
 {
     if (f.n == 0) return 0;
     if (f.n >= kMaxPairTargets) return -7;
-    SPH_LAUNCH_PAIRS(k_reinit, f.n, bt, f, w, s);
+    SPH_LAUNCH_PAIRS(k_reinit, f.n, f.list ? part_blocks(f.n, kPartNear, f.block) : 0, bt, f, w, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
