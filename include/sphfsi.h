@@ -407,11 +407,10 @@ typedef struct {
                               a row (at most 64 in 2-D, 128 in 3-D; a fuller row falls back to the
                               cell visit for that particle), and stream the rows in momentum,
                               continuity and reinitialisation; not with tiles or cell_reach 2
-                              (default 1 in 3-D from 262 144 particles in the context, else 0) */
-    int32_t list_lanes;    /* threads per fluid particle of the row build: 1 (one warp per cell,
-                              each candidate loaded once for the cell's particles), 8, 16 or 32
-                              (default 8 in 2-D, 1 in 3-D; 0 keeps the current value); all build
-                              the same rows */
+                              (default 1 from 16 384 fluid particles in the context in 3-D and
+                              32 768 in 2-D, else 0) */
+    int32_t list_lanes;    /* 1, 8, 16 or 32 (default 1; 0 keeps the current value): kept for
+                              callers that set it; one row build, a warp per cell, serves them all */
 } sphfsi_tuning;
 
 /* Set or read the launch shape (SPHFSI_E_INVAL for values outside the lists). */
@@ -422,10 +421,8 @@ int sphfsi_get_tuning(sphfsi_ctx *c, sphfsi_tuning *t);
  * workload: for each candidate setting, `steps` graph-replayed steps of size
  * dt_F (as sphfsi_run) to warm up, then `steps` timed with CUDA events.  The
  * search goes over the lane count (block 128), then the pair-loop form,
- * then neighbour rows on or off (with rows: the row build's lane count),
- * then (without rows) tiles on or off and the row form, then the block
- * size, then the
- * records form, then (2-D with a solid) the solid kernel variant, keeping the
+ * then neighbour rows on or off, then (without rows) tiles on or off and the
+ * row form, then the block size, then the records form, then (2-D with a solid) the solid kernel variant, keeping the
  * fastest of each.
  * Every device allocation of the context is saved before and restored after
  * each trial and at the end, so the simulation state, time and counters are

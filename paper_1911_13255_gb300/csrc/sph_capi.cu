@@ -148,6 +148,7 @@ struct sphfsi_ctx {
     bool profiling = false;
     cudaEvent_t ev[kEvents] = {};
     int kernels_per_step = 0;
+    bool fork_first = false;   // the solid branch starts before the neighbour rows are built
     int max_reach = 1;   // largest cell reach of the instances (sphfsi_params::cell_reach)
     // side stream for the solid branch, which runs beside momentum and continuity
     cudaStream_t side = nullptr;
@@ -280,6 +281,30 @@ int mark(sphfsi_ctx *c, int k, cudaStream_t st)
 }
 int mark(sphfsi_ctx *c, int k) { return mark(c, k, c->st); }
 
+// sub-steps of an instance's first step from rest (Eqs. dt-relax, dts-advection),
+// for the launch-shape defaults
+double first_substeps(const InstHost &h)
+{
+    if (h.ns == 0) return 0.0;
+    const double cS = std::sqrt(h.s_E / (3.0 * (1.0 - 2.0 * h.s_nu)) / h.s_rho0);
+    return std::floor((h.f_dp / h.f_c0) / (h.s_dp / cS)) + 1.0;
+}
+
+// the pair loops' cell form at its default launch shape
+void cell_form(const sphfsi_ctx *c, Fluid &F)
+{
+    const bool small = F.n + c->S.n < 262144;
+    // small problems are latency-bound: 8 lanes per target and direct pair
+    // evaluation (dam break: 0.105 -> 0.102 ms per step), neighbour cells a row
+    // at a time (rows of cells are built for cells of >= 2 h_F); large 2-D
+    // problems are issue-bound: 4 lanes and compacted pairs; 3-D: 8 lanes below
+    // 200 000 fluid particles, else 4, direct pairs
+    F.list = 0;
+    F.lanes = c->dim == 2 ? (small ? 8 : 4) : (F.n < 200000 ? 8 : 4);
+    F.compact = c->dim == 2 && !small ? 1 : 0;
+    F.rows = small && c->max_reach == 1 ? 1 : 0;
+}
+
 int enqueue_step(sphfsi_ctx *c, double dt)
 {
     cudaStream_t st = c->st;
@@ -290,11 +315,16 @@ int enqueue_step(sphfsi_ctx *c, double dt)
     // (r^n) binning, counting sort and FP32 records
     TRY(launch_bin_all(c->bt, c->F, c->S, D, 1, dt > 0.0 ? dt : 0.0, c->K_fixed, st));
     TRY(mark(c, 2));
-    // neighbour rows of the pair loops (rebuild steps, when on)
-    TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
+    // neighbour rows of the pair loops (rebuild steps, when on) and a3, the
+    // density reinitialisation (no-op on other steps).  Where the solid branch
+    // is the longer one (fork_first) the rows wait until it has started: the
+    // reinitialisation, which it waits for, then visits the cells.
+    const bool late_rows = c->F.list && c->fork_first && c->S.n;
+    Fluid cells = c->F;
+    if (late_rows) cell_form(c, cells);
+    else TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
     TRY(mark(c, 1));
-    // a3: density reinitialisation (no-op on other steps)
-    TRY(launch_reinit(c->bt, c->F, c->W, c->S, D, st));
+    TRY(launch_reinit(c->bt, late_rows ? cells : c->F, c->W, c->S, D, st));
     TRY(mark(c, 3));
     // The solid branch (a5, then a7 + a8) depends only on the records written
     // so far, so it runs on the side stream while the main stream does a4
@@ -314,6 +344,7 @@ int enqueue_step(sphfsi_ctx *c, double dt)
         TRY(mark(c, 8, c->side));
         TRY(cuda_rc(cudaEventRecord(c->join_ev, c->side)));
     }
+    if (late_rows) TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
     TRY(launch_momentum(c->bt, c->F, c->W, c->S, D, st));
     TRY(mark(c, 5));
     TRY(launch_density(c->bt, c->F, c->W, c->S, D, st));
@@ -897,14 +928,8 @@ int sphfsi_finalize(sphfsi_ctx *c)
     // ---- fluid
     Fluid &F = c->F;
     F.n = (int)nf;
-    // small problems are latency-bound: 8 lanes per target and direct pair
-    // evaluation (dam break: 0.105 -> 0.102 ms per step); large 2-D problems
-    // are issue-bound: 4 lanes and compacted pairs; 3-D: 8 lanes below 200 000
-    // fluid particles, else 4, direct pairs
     const bool small = nf + ns < 262144;
-    F.lanes = D == 2 ? (small ? 8 : 4) : (nf < 200000 ? 8 : 4);
     F.block = 128;
-    F.compact = D == 2 && !small ? 1 : 0;
     F.tile = 0;
     // records from the cell groups for small problems (one launch fewer),
     // one thread per slot for large ones (no idle lanes)
@@ -913,9 +938,6 @@ int sphfsi_finalize(sphfsi_ctx *c)
     // than the four kernels with programmatic launches (dam break: binning
     // 35.4 vs 31.2 us): off by default
     F.bin_fused = 0;
-    // neighbour cells a row at a time where latency, not issue, bounds the loops
-    // (rows and tiles are built for cells of >= 2 h_F)
-    F.rows = small && c->max_reach == 1 ? 1 : 0;
     F.reach = c->max_reach;
     // tiles: T cells of a grid row per block (16 in 2-D, 4 in 3-D); the
     // staging area holds about three times the mean neighbourhood
@@ -981,13 +1003,34 @@ int sphfsi_finalize(sphfsi_ctx *c)
     TRY(dalloc(c, &F.bsum, 4096));
     TRY(dalloc(c, &F.gbar, 2));
     // neighbour rows (tuned): about 20 (2-D) or 80 (3-D) neighbours per fluid
-    // particle on a lattice, wall neighbours included.  On by default for
-    // large 3-D problems (3-D duct, 3M fluid: momentum 6.2 -> 2.4 ms,
-    // continuity 4.9 -> 1.65 ms for a 2.4 ms row build); off for 2-D, where
-    // the row build costs more than it saves (dam break 0.100 -> 0.107 ms)
-    F.list = D == 3 && !small ? 1 : 0;
-    if (F.list) F.compact = 0;
-    F.list_lanes = D == 2 ? 8 : 1;
+    // particle on a lattice, wall neighbours included.  On from 32 768 fluid
+    // particles in 2-D (2 lanes per target) and 16 384 in 3-D (4): below, the
+    // loops are too short to pay for the build.  Step with the cell form and
+    // with rows: 2-D channels of 10k, 40k and 79k particles 67, 80 and 146 us
+    // against 62, 76 and 108; batches of 28k, 171k and 577k 130, 248 and 574
+    // against 138, 234 and 485; 3-D tanks of 6k, 17k, 62k and 175k 230, 257, 393
+    // and 780 against 241, 246, 320 and 476.
+    F.n = (int)nf;
+    c->S.n = (int)ns;
+    cell_form(c, F);
+    if (c->max_reach == 1 && nf >= (D == 3 ? 16384 : 32768)) {
+        F.list = 1;
+        F.lanes = D == 3 ? 4 : 2;
+        F.compact = 0;
+        F.rows = 0;
+    }
+    // Is the solid branch longer than rows, momentum and continuity?  From the
+    // first step's K and the measured cost of a sub-step (about 2 us in one
+    // cluster, 5 us in the 2-D window kernel, 8 us in 3-D) against 25 us and 1 ns
+    // per fluid particle in 2-D, 2.5 ns in 3-D.  Dam break of 56k particles and a
+    // body of 6400, 25 sub-steps: step 199 us with the rows first, 185 so.
+    {
+        double K = 0.0;
+        for (int b = 0; b < B; b++) K = std::max(K, first_substeps(c->ih[b]));
+        const double sub = D == 3 ? 8.0 : (max_ns > 2048 ? 5.0 : 2.0);
+        c->fork_first = sub * K > 25.0 + (D == 3 ? 2.5e-3 : 1e-3) * (double)nf;
+    }
+    F.list_lanes = 1;
     F.list_cap = D == 2 ? 64 : 128;
     TRY(dalloc(c, &F.nbl, (size_t)nf * F.list_cap));
     TRY(dalloc(c, &F.nbc, nf));
@@ -2008,13 +2051,6 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
         if (!rc && c->max_reach == 1) {
             cur.list = 1 - cur.list;
             if (cur.list) cur.tile = 0;
-            rc = consider(cur);
-        }
-        cur = *best;
-        for (int k = 0; k < 3 && !rc && cur.list; k++) {
-            const int ll[3] = {1, 8, 32};
-            if (ll[k] == best->list_lanes) continue;
-            cur.list_lanes = ll[k];
             rc = consider(cur);
         }
         cur = *best;

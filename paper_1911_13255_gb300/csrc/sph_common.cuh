@@ -210,7 +210,7 @@ struct Fluid {
     // are kept as entries idx << 7 | cell-offset code in row i of list_cap
     // entries; the pair loops stream the rows.  nbc[i] = nF | nW << 11 | flags.
     int list;
-    int list_lanes;     // threads per target of the row build (8, 16 or 32; tuned)
+    int list_lanes;     // sphfsi_tuning::list_lanes as set (one row build serves every value)
     int list_cap;
     uint32_t *nbl;
     uint32_t *nbc;

@@ -29,7 +29,7 @@ __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, con
         const float vi[3] = {Wi.x, Wi.y, Wi.z};
         const float drhoi = Wi.w, rhoi = P.rho0 + Wi.w;
         int cx, cy, cz;
-        cell_xyz(f.cell_of[i], In, cx, cy, cz);
+        cell_xyz<D>(f.cell_of[i], In, cx, cy, cz);
         const float inv2c0 = 0.5f / P.c0;
         auto none = [](int, float, float, float) {};
         fluid_pairs<D, L, CP, FORM, kFluidOnly, true>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, P.rc2F, list, stride, ts,
@@ -211,7 +211,7 @@ __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, cons
     if (act) {
         const float4 Pi = f.P4[i], Li = f.L4[i];
         int cx, cy, cz;
-        cell_xyz(f.cell_of[i], In, cx, cy, cz);
+        cell_xyz<D>(f.cell_of[i], In, cx, cy, cz);
         auto wall_pair = [&](int q, float ox, float oy, float oz) {
             float d[3];
             const float4 Aq = w.A4[q];

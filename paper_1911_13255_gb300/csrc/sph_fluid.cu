@@ -35,7 +35,7 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
         const float vi[3] = {Vi.x, Vi.y, Vi.z};
         const float rhoi = P.rho0 + Vi.w, pi = Pi.w;
         int cx, cy, cz;
-        cell_xyz(f.cell_of[i], In, cx, cy, cz);
+        cell_xyz<D>(f.cell_of[i], In, cx, cy, cz);
         const float c0 = P.c0, eta2 = 2.0f * P.eta;
         // walls (v~ = a~ = 0) and solid particles at their start-of-step
         // positions with v~, a~
@@ -173,16 +173,12 @@ int launch_momentum(const Batch &bt, const Fluid &f, const Walls &w, const Solid
 
 // ---------------------------------------------------------------------------
 // a2 (neighbour rows): each fluid target's in-support fluid neighbours (from
-// the front of its row) and in-support wall neighbours (from the back),
-// over the 3^(d-1) rows of three cells around its cell (a row's cells are
-// consecutive in the cell-sorted records, so its candidates are one flat
-// range), with the pair loops' own FP32 test on the records, and whether a
-// neighbour cell holds solid particles.  L lanes per target test 2 L
-// candidates a round (both loads issued first); the in-support ones get their
-// places by ballots over the L lanes, so a row lists its entries in the
-// candidate order whatever L is.  Entries that do not fit are dropped and the
-// row is marked overflowed (its target then takes the cell form; every
-// write stays inside the row).  Runs on rebuild steps.
+// the front of its row) and in-support wall neighbours (from the back), in
+// the order of the 3^d cells around its cell, with the pair loops' own FP32
+// test on the records, and whether a neighbour cell holds solid particles.
+// Entries that do not fit are dropped and the row is marked overflowed (its
+// target then takes the cell form; every write stays inside the row).  Runs on
+// rebuild steps.
 // ---------------------------------------------------------------------------
 // Row i's word; a row with boundary neighbours, or one that overflowed, also
 // enters the list of its kind, one atomic per warp and kind (the order of a
@@ -205,156 +201,210 @@ __device__ __forceinline__ void row_word(const Fluid &f, int i, int nF, int nW, 
     }
 }
 
-template <int D, int L>
-__global__ void __launch_bounds__(kMaxBlock) k_pairlist(Batch bt, Fluid f, Walls w, Solid s)
+// One warp per cell, in two stages:
+//  - the candidates of the 3^d cells around it, 32 at a time, are tested
+//    against the bounding box of the cell's particles (a coalesced load and a
+//    ballot) and the ones within reach of it, about 60 % of them, are kept in
+//    shared memory in candidate order;
+//  - up to kCand of them per lane go to registers, and every particle of the cell is
+//    tested against 32 of them per step; a ballot gives the in-support ones
+//    consecutive places in its row.
+// What bounds a row build is instruction issue over the candidate tests (475
+// per particle in 3-D, 61 in 2-D).  With one lane per particle of the cell, as
+// this build had it before, 20 to 45 % of the lanes idled (cells of 8 to 18
+// particles), every candidate was tested, and each append stored 4 bytes to as
+// many rows as lanes; with 8 lanes per particle every particle loaded its
+// candidates itself.  Here all lanes test, and a row is written in runs.
+// Measured (lane per particle, 8 lanes per particle, this): 3-D duct, 3.0M
+// particles, 2052, -, 1172 us; 375k 394, 739, 164 us; 3-D tank, 62k 168, 144,
+// 47 us; batch of 32 2-D channels, 577k 124, 234, 109 us; 2-D channel, 10k 22,
+// 14, 12 us.  3-D: 127M warp instructions on the 375k duct against 227M, issue
+// 65 % active; 4 candidates per lane (96 registers) beat 6 (1714 us on 3.0M) and
+// a cap of 80 registers (1290 us).
+// The in-support test is the pair loops' own (rel_d on the records).
+template <int D> constexpr int kCand = D == 3 ? 4 : 2;   // candidates per lane and batch
+constexpr int kRowWarps = 4;
+
+template <int D>
+struct RowWarp {
+    float4 cand[32 * (kCand<D> + 1)];   // position in its own cell, entry bits
+    float4 target[32];
+};
+
+__device__ __forceinline__ unsigned ordered_bits(float x)
 {
-    pdl_enter();
-    if (step_failed(bt)) return;   // the step's cell starts are not valid
-    if (!rebuild_step(bt, f)) return;   // held configuration: the rows stay
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = t / L, lane = t % L;
-    if (i >= f.n) return;   // the L lanes of a target leave together
-    const int wl = threadIdx.x & 31;
-    const unsigned gmask = L == 32 ? 0xffffffffu : ((1u << L) - 1u) << (wl & ~(L - 1));
-    const unsigned below = (1u << wl) - 1u;
-    const Inst &In = bt.I[f.inst[i]];
-    const Grid &g = In.g;
-    const float rc2 = In.P.rc2F;
-    const float4 Pi = f.P4[i];
-    int cx, cy, cz;
-    cell_xyz(f.cell_of[i], In, cx, cy, cz);
-    uint32_t *row = f.nbl + (size_t)i * f.list_cap;
-    const int cap = f.list_cap;
-    int nF = 0, nW = 0;
-    bool solid = false;
-    // every loop bound below is the same for the L lanes of the target
-    for_each_row<D>(g, In.c0, cx, cy, cz, [&](const int c[3], float oy, float oz, int code0) {
-        const Row3 rf = row_of(f.cstart, c);
-        const Row3 rw = row_of(w.cstart, c);
-        if (s.n) solid = solid || row_of(s.cstart, c).n > 0;
-        for (int qb = 0; qb < rf.n; qb += 2 * L) {
-            const int q0 = qb + lane, q1 = q0 + L;
-            int k0 = 0, k1 = 0;
-            const int j0 = q0 < rf.n ? row_slot(rf, q0, k0) : -1;
-            const int j1 = q1 < rf.n ? row_slot(rf, q1, k1) : -1;
-            const float4 P0 = j0 >= 0 ? f.P4[j0] : Pi;
-            const float4 P1 = j1 >= 0 ? f.P4[j1] : Pi;
-            float d[3];
-            const bool in0 = j0 >= 0 && j0 != i && rel_d<D>(Pi, P0, row_ox(k0, g), oy, oz, d) < rc2;
-            const bool in1 = j1 >= 0 && j1 != i && rel_d<D>(Pi, P1, row_ox(k1, g), oy, oz, d) < rc2;
-            const unsigned m0 = __ballot_sync(gmask, in0) & gmask;
-            const unsigned m1 = __ballot_sync(gmask, in1) & gmask;
-            const int n0 = __popc(m0);
-            if (in0) {
-                const int q = nF + __popc(m0 & below);
-                if (q < cap) row[q] = ((uint32_t)j0 << kCodeBits) | row_code(code0 + k0);
-            }
-            if (in1) {
-                const int q = nF + n0 + __popc(m1 & below);
-                if (q < cap) row[q] = ((uint32_t)j1 << kCodeBits) | row_code(code0 + k1);
-            }
-            nF += n0 + __popc(m1);
-        }
-        for (int qb = 0; qb < rw.n; qb += L) {
-            const int q0 = qb + lane;
-            int k0 = 0;
-            const int a = q0 < rw.n ? row_slot(rw, q0, k0) : -1;
-            float d[3];
-            const bool in = a >= 0 && rel_d<D>(Pi, w.A4[a], row_ox(k0, g), oy, oz, d) < rc2;
-            const unsigned m = __ballot_sync(gmask, in) & gmask;
-            if (in) {
-                const int q = cap - 1 - (nW + __popc(m & below));
-                if (q >= 0) row[q] = ((uint32_t)a << kCodeBits) | row_code(code0 + k0);
-            }
-            nW += __popc(m);
-        }
-    });
-    if (lane == 0) row_word(f, i, nF, nW, solid);
+    const unsigned u = __float_as_uint(x);
+    return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float from_ordered(unsigned u)
+{
+    return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
 }
 
-// The same rows built per cell, one lane per particle of the cell: each lane
-// appends to its own row, so the entries come in the same order as above
-// (fluid by cell, then slot, from the front; walls likewise from the back).
-// The rows of the targets [t0, t1) of one non-empty cell, G lanes of a
-// group per round (this thread is lane `lane` of its group): every
-// candidate of the 3^d neighbour cells is loaded once for the group and each
-// lane tests its own target against it.  No warp-wide operation, so the two
-// half-warps of a warp may run two cells side by side.
-template <int D>
-__device__ __forceinline__ void cell_rows(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int cell,
-                                          int t0, int t1, int lane, int G)
+// Tests the nt targets (slots t0 ..) against the m candidates of the buffer, NR
+// of them per lane (straight-line code: the NR tests of a target overlap), and
+// appends to their rows; lane t holds target t's count.  WALL: rows are filled
+// from the back; otherwise the target itself is left out (entry `self` with
+// its slot).
+template <int D, bool WALL, int NR>
+__device__ __forceinline__ void row_tests(const Fluid &f, const Grid &g, float rc2, const RowWarp<D> &sw, int m, int t0,
+                                          int nt, int lane, uint32_t self, int &count)
 {
-    const Inst &In = bt.I[f.inst[t0]];
-    const Grid &g = In.g;
-    const float rc2 = In.P.rc2F;
+    float4 c[NR];
+    float o[NR][3];
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+        const int k = 32 * r + lane;
+        // no candidate: too far for every target
+        c[r] = k < m ? sw.cand[k] : make_float4(1e30f, 1e30f, 1e30f, __uint_as_float(0u));
+        row_offset(__float_as_uint(c[r].w), g, o[r][0], o[r][1], o[r][2]);
+    }
+    const unsigned below = (1u << lane) - 1u;
     const int cap = f.list_cap;
-    int cx, cy, cz;
-    cell_xyz(cell, In, cx, cy, cz);
-    for (int tb = t0; tb < t1; tb += G) {
-        const int i = tb + lane;
-        const bool act = i < t1;
-        const float4 Pi = f.P4[act ? i : t0];
-        uint32_t *row = f.nbl + (size_t)(act ? i : t0) * cap;
-        int nF = 0, nW = 0;
-        bool solid = false;
-        for_each_cell<D, 1>(g, In.c0, cx, cy, cz, [&](int c, float ox, float oy, float oz, int code) {
-            const uint32_t rc = row_code(code);
-            const int j1 = f.cstart[c + 1];
-#pragma unroll 4
-            for (int j = f.cstart[c]; j < j1; j++) {
-                float d[3];
-                const bool in = rel_d<D>(Pi, f.P4[j], ox, oy, oz, d) < rc2 && j != i && act;
-                if (in) {
-                    if (nF < cap) row[nF] = ((uint32_t)j << kCodeBits) | rc;
-                    nF++;
-                }
-            }
-            const int a1 = w.cstart[c + 1];
-            for (int a = w.cstart[c]; a < a1; a++) {
-                float d[3];
-                const bool in = rel_d<D>(Pi, w.A4[a], ox, oy, oz, d) < rc2 && act;
-                if (in) {
-                    if (nW < cap) row[cap - 1 - nW] = ((uint32_t)a << kCodeBits) | rc;
-                    nW++;
-                }
-            }
-            if (s.n && s.cstart[c + 1] > s.cstart[c]) solid = true;
-        });
-        if (act) row_word(f, i, nF, nW, solid);
+    uint32_t *row = f.nbl + (size_t)t0 * cap + (WALL ? cap - 1 : 0);
+    uint32_t me = ((uint32_t)t0 << kCodeBits) | self;
+#pragma unroll 1
+    for (int t = 0; t < nt; t++, row += cap, me += 1u << kCodeBits) {
+        const float4 P = sw.target[t];
+        int base = __shfl_sync(0xffffffffu, count, t);
+        unsigned hit[NR];
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+            float d[3];
+            const bool in = rel_d<D>(P, c[r], o[r][0], o[r][1], o[r][2], d) < rc2 &&
+                            (WALL || __float_as_uint(c[r].w) != me);
+            hit[r] = __ballot_sync(0xffffffffu, in);
+        }
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+            const int q = base + __popc(hit[r] & below);
+            if ((hit[r] >> lane & 1u) && q < cap) row[WALL ? -q : q] = __float_as_uint(c[r].w);
+            base += __popc(hit[r]);
+        }
+        if (lane == t) count = base;
     }
 }
 
-// One warp per two consecutive cells.  When they hold at most 32 targets
-// together, one round builds both: the first cell's targets take the first
-// lanes, the second cell's the next ones (in the 3-D duct, cells of 8, 12
-// and 18 particles come in rows where such pairs are common, and the two
-// groups then walk neighbour cells of nearly equal size); otherwise the
-// whole warp builds one cell after the other.  Either way each target's row
-// is built by one lane in candidate order, so the rows do not depend on the
-// grouping.
-// 16 resident blocks per SM (32 registers a thread): the build is issue- and
-// load-latency bound, and the extra warps outweigh a few spilled registers
-// (3-D duct: 2.37 -> 2.32 ms; 56-register pair loops, by contrast, ran
-// slower than at 64).
-template <int D>
-__global__ void __launch_bounds__(128, 16) k_pairlist_cells(Batch bt, Fluid f, Walls w, Solid s)
+template <int D, bool WALL>
+__device__ __forceinline__ void row_batch(const Fluid &f, const Grid &g, float rc2, const RowWarp<D> &sw, int m, int t0,
+                                          int nt, int lane, uint32_t self, int &count)
 {
+    const int n = (m + 31) >> 5;
+    if constexpr (D == 3) {
+        if (n == 4) row_tests<D, WALL, 4>(f, g, rc2, sw, m, t0, nt, lane, self, count);
+        else if (n == 3) row_tests<D, WALL, 3>(f, g, rc2, sw, m, t0, nt, lane, self, count);
+    }
+    if (n == 2) row_tests<D, WALL, 2>(f, g, rc2, sw, m, t0, nt, lane, self, count);
+    else if (n == 1) row_tests<D, WALL, 1>(f, g, rc2, sw, m, t0, nt, lane, self, count);
+}
+
+template <int D>
+__global__ void __launch_bounds__(32 * kRowWarps, D == 3 ? 5 : 8) k_pairlist_cells(Batch bt, Fluid f, Walls w, Solid s)
+{
+    __shared__ RowWarp<D> s_warp[kRowWarps];
     pdl_enter();
     if (step_failed(bt)) return;   // the step's cell starts are not valid
     if (!rebuild_step(bt, f)) return;
-    const int c0 = 2 * (blockIdx.x * 4 + (int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
-    if (c0 >= bt.ncell) return;
-    const bool two = c0 + 1 < bt.ncell;
-    const int a0 = f.cstart[c0], a1 = f.cstart[c0 + 1];   // the second cell starts where the first ends
-    const int b1 = two ? f.cstart[c0 + 2] : a1;
-    const int na = a1 - a0;
-    if (b1 - a0 <= 32) {
-        const bool second = lane >= na;
-        const int t0 = second ? a1 : a0, t1 = second ? b1 : a1, ll = second ? lane - na : lane;
-        if (ll < t1 - t0) cell_rows<D>(bt, f, w, s, second ? c0 + 1 : c0, t0, t1, ll, 32);
-    } else {
-        if (a0 < a1) cell_rows<D>(bt, f, w, s, c0, a0, a1, lane, 32);
-        if (a1 < b1) cell_rows<D>(bt, f, w, s, c0 + 1, a1, b1, lane, 32);
+    const int cell = blockIdx.x * kRowWarps + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (cell >= bt.ncell) return;
+    const int a0 = f.cstart[cell], a1 = f.cstart[cell + 1];
+    if (a0 >= a1) return;
+    RowWarp<D> &sw = s_warp[threadIdx.x >> 5];
+    const Inst &In = bt.I[f.inst[a0]];
+    const Grid &g = In.g;
+    const float rc2 = In.P.rc2F, reach2 = rc2 * 1.0001f;   // the box test's rounding stays within the margin
+    constexpr int NR = D == 3 ? 9 : 3;
+    constexpr uint32_t self = 1u | 1u << 2 | 1u << 4;   // the code of the target's own cell
+    // lane r < NR: row r's three cells in the fluid, wall and solid sets
+    Row3 mf{0, 0, 0, 0, 0, 0}, mw = mf;
+    bool solid = false;
+    {
+        int cx, cy, cz;
+        cell_xyz<D>(cell, In, cx, cy, cz);
+        const int dy = lane % 3 - 1, dz = D == 3 ? lane / 3 - 1 : 0;
+        const int y = cy + dy, z = cz + dz;
+        if (lane < NR && y >= 0 && y < g.nc[1] && z >= 0 && z < g.nc[2]) {
+            const int base = In.c0 + g.nc[0] * (y + g.nc[1] * z);
+            int c[3];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                int x = cx + k - 1;
+                if (x < 0 || x >= g.nc[0]) x = g.periodic_x ? (x < 0 ? x + g.nc[0] : x - g.nc[0]) : -1;
+                c[k] = x < 0 ? -1 : base + x;
+            }
+            mf = row_of(f.cstart, c);
+            mw = row_of(w.cstart, c);
+            if (s.n) solid = row_of(s.cstart, c).n > 0;
+        }
+        solid = __any_sync(0xffffffffu, solid);
+    }
+    for (int t0 = a0; t0 < a1; t0 += 32) {
+        const int nt = min(32, a1 - t0);
+        const float4 P = f.P4[t0 + (lane < nt ? lane : 0)];
+        __syncwarp();
+        sw.target[lane] = P;
+        float lo[3], hi[3];
+        {
+            const float p[3] = {P.x, P.y, P.z};
+#pragma unroll
+            for (int k = 0; k < D; k++) {
+                lo[k] = from_ordered(__reduce_min_sync(0xffffffffu, ordered_bits(p[k])));
+                hi[k] = from_ordered(__reduce_max_sync(0xffffffffu, ordered_bits(p[k])));
+            }
+        }
+        int nF = 0, nW = 0;   // of target `lane`
+        auto gather = [&](const Row3 &mine, const float4 *__restrict__ rec, auto wall, int &count) {
+            constexpr bool WALL = decltype(wall)::value;
+            int m = 0;
+            for (int r = 0; r < NR; r++) {
+                Row3 row;
+                row.n = __shfl_sync(0xffffffffu, mine.n, r);
+                if (row.n == 0) continue;
+                row.a0 = __shfl_sync(0xffffffffu, mine.a0, r);
+                row.a1 = __shfl_sync(0xffffffffu, mine.a1, r);
+                row.a2 = __shfl_sync(0xffffffffu, mine.a2, r);
+                row.n0 = __shfl_sync(0xffffffffu, mine.n0, r);
+                row.n01 = __shfl_sync(0xffffffffu, mine.n01, r);
+                const float oy = (float)(1 - r % 3) * g.csf[1], oz = D == 3 ? (float)(1 - r / 3) * g.csf[2] : 0.0f;
+                const uint32_t code = (uint32_t)(r % 3) << 2 | (D == 3 ? (uint32_t)(r / 3) : 1u) << 4;
+                for (int q0 = 0; q0 < row.n; q0 += 32) {
+                    const int q = q0 + lane;
+                    int k;
+                    const int j = row_slot(row, q < row.n ? q : 0, k);
+                    const float4 X = rec[j];
+                    // distance of the candidate, in the target cell's frame, from the box
+                    const float x = X.x - row_ox(k, g), y = X.y - oy;
+                    const float ex = fmaxf(fmaxf(lo[0] - x, x - hi[0]), 0.0f);
+                    const float ey = fmaxf(fmaxf(lo[1] - y, y - hi[1]), 0.0f);
+                    float e2 = ex * ex + ey * ey;
+                    if (D == 3) {
+                        const float z = X.z - oz;
+                        const float ez = fmaxf(fmaxf(lo[2] - z, z - hi[2]), 0.0f);
+                        e2 += ez * ez;
+                    }
+                    const bool keep = q < row.n && e2 < reach2;
+                    const unsigned mk = __ballot_sync(0xffffffffu, keep);
+                    if (keep)
+                        sw.cand[m + __popc(mk & ((1u << lane) - 1u))] =
+                            make_float4(X.x, X.y, X.z, __uint_as_float(((uint32_t)j << kCodeBits) | code | (uint32_t)k));
+                    m += __popc(mk);
+                    if (m >= 32 * kCand<D>) {
+                        __syncwarp();
+                        row_batch<D, WALL>(f, g, rc2, sw, 32 * kCand<D>, t0, nt, lane, self, count);
+                        m -= 32 * kCand<D>;
+                        const float4 rest = sw.cand[32 * kCand<D> + lane];
+                        __syncwarp();
+                        if (lane < m) sw.cand[lane] = rest;
+                    }
+                }
+            }
+            __syncwarp();
+            row_batch<D, WALL>(f, g, rc2, sw, m, t0, nt, lane, self, count);
+            __syncwarp();
+        };
+        gather(mf, f.P4, std::false_type{}, nF);
+        if (__any_sync(0xffffffffu, mw.n > 0)) gather(mw, w.A4, std::true_type{}, nW);
+        if (lane < nt) row_word(f, t0 + lane, nF, nW, solid);
     }
 }
 
@@ -362,22 +412,9 @@ int launch_pairlist(const Batch &bt, const Fluid &f, const Walls &w, const Solid
 {
     if (f.n == 0 || !f.list) return 0;
     if (f.n >= kMaxPairTargets || w.n >= kMaxPairTargets) return -7;
-    // its own lane count: wide groups load a row's consecutive candidates together
-    auto go = [&](auto Dc, auto Lc) {
-        constexpr int D_ = decltype(Dc)::value, L_ = decltype(Lc)::value;
-        launch_k(k_pairlist<D_, L_>, grid_blocks(f.n, L_, 128), 128, 0, st, bt, f, w, s);
-    };
-    auto by_lanes = [&](auto Dc) {
-        constexpr int D_ = decltype(Dc)::value;
-        if (f.list_lanes == 1) launch_k(k_pairlist_cells<D_>, (bt.ncell + 7) / 8, 128, 0, st, bt, f, w, s);
-        else if (f.list_lanes == 8) go(Dc, std::integral_constant<int, 8>{});
-        else if (f.list_lanes == 16) go(Dc, std::integral_constant<int, 16>{});
-        else if (f.list_lanes == 32) go(Dc, std::integral_constant<int, 32>{});
-        else return false;
-        return true;
-    };
-    const bool ok = dim == 2 ? by_lanes(std::integral_constant<int, 2>{}) : by_lanes(std::integral_constant<int, 3>{});
-    if (!ok) return -1;
+    const unsigned grid = (unsigned)((bt.ncell + kRowWarps - 1) / kRowWarps);
+    if (dim == 2) launch_k(k_pairlist_cells<2>, grid, 32 * kRowWarps, 0, st, bt, f, w, s);
+    else launch_k(k_pairlist_cells<3>, grid, 32 * kRowWarps, 0, st, bt, f, w, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -403,7 +440,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_solid_fluid_force(Batch bt, Fl
     if (act) {
         const float4 A = s.A4[k], VB = s.VB4[k], AB = s.AB4[k], N = s.N4[k];
         int cx, cy, cz;
-        cell_xyz(s.cell_of[k], In, cx, cy, cz);
+        cell_xyz<D>(s.cell_of[k], In, cx, cy, cz);
         auto pair = [&](int j, float ox, float oy, float oz) {
             const float4 Pj = f.P4[j];
             // the fluid side sees this pair with the opposite cell offset
@@ -512,7 +549,7 @@ __global__ void k_debug_pairs(Batch bt, Fluid f, Walls w, Solid s, int inst, int
         key = f.cell_of[k];
     }
     int cx, cy, cz;
-    cell_xyz(key, In, cx, cy, cz);
+    cell_xyz<D>(key, In, cx, cy, cz);
     int cnt = 0;
     int base = out ? offs[row] : 0;
     auto visit = [&](int c, float, float, float, int) {

@@ -686,14 +686,16 @@ __device__ __forceinline__ float eos_dp(float drho_i, float drho_j, const Phys &
     return P.p_coef * ((drho_i - drho_j) * inv) * s;
 }
 
-// local cell coordinates of a global cell index
+// local cell coordinates of a global cell index (integer divisions are long
+// instruction sequences: one per axis beyond the first)
+template <int D>
 __device__ __forceinline__ void cell_xyz(int gkey, const Inst &In, int &cx, int &cy, int &cz)
 {
     const Grid &g = In.g;
-    const int key = gkey - In.c0;
-    cx = key % g.nc[0];
-    cy = (key / g.nc[0]) % g.nc[1];
-    cz = key / (g.nc[0] * g.nc[1]);
+    const int key = gkey - In.c0, q = key / g.nc[0];
+    cx = key - q * g.nc[0];
+    cz = D == 3 ? q / g.nc[1] : 0;
+    cy = q - cz * g.nc[1];
 }
 
 // Fluid-solid (or fluid-wall) pair: force on the fluid particle divided by
