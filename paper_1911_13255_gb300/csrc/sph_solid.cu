@@ -1895,7 +1895,8 @@ static int launch_solid_window(const Batch &bt, const Solid &s, int dim, cudaStr
 
 // 3-D bodies above this size take the windowed kernel instead of the cluster
 // kernel, whose lanes read every neighbour's three Q rows across the cluster
-constexpr int kWin3dFrom = 2048;
+// (plate of 1408 particles, 10 sub-steps: 172 -> 92 us beside the fluid loops)
+constexpr int kWin3dFrom = 512;
 
 int launch_solid_substeps(const Batch &bt, Solid &s, const Phys &P0, int dim, int *path, cudaStream_t st)
 {
