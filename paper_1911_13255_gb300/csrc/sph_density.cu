@@ -30,23 +30,21 @@ __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, con
         const float drhoi = Wi.w, rhoi = P.rho0 + Wi.w;
         int cx, cy, cz;
         cell_xyz<D>(f.cell_of[i], In, cx, cy, cz);
-        const float inv2c0 = 0.5f / P.c0;
+        const float half_inv_h = 0.5f * P.inv_hF, mdW = P.mF * (P.dWcF * P.inv_hF);   // as in momentum_one
+        const EosDiff dp(drhoi, P);
         auto none = [](int, float, float, float) {};
         fluid_pairs<D, L, CP, FORM, kFluidOnly, true>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, P.rc2F, list, stride, ts,
                                 [&](int j) { return f.W4[j]; },
                                 [&](int, const float4 &, const float4 &Wj, const float *d, float r2, float, float,
                                     float) {
-                if (r2 == 0.0f) return;   // a clumped pair: no direction, dW(0) = 0
+                if (!(r2 >= kMinNormal)) return;   // a clumped pair: no direction, dW(0) = 0
                 const float rhoj = P.rho0 + Wj.w;
-                // one reciprocal square root for 1/r and r (r2 > 0 here)
-                const float invr = rsqrtf(r2), r = r2 * invr;
-                float dW = dW_F(r, P);
-                float UL = -(vi[0] * d[0] + vi[1] * d[1] + (D == 3 ? vi[2] * d[2] : 0.0f)) * invr;
-                float UR = -(Wj.x * d[0] + Wj.y * d[1] + (D == 3 ? Wj.z * d[2] : 0.0f)) * invr;
-                float rb = 0.5f * (rhoi + rhoj);
-                // (v_i - v~_ij).grad_i W = -dW (U_L - U*), U* = (U_L + U_R)/2 + (p_i - p_j) / (2 rho c0)
-                float diff = 0.5f * (UL - UR) - eos_dp(drhoi, Wj.w, P) * inv2c0 / rb;
-                rate += __fdividef(P.mF, rhoj) * (-dW) * diff;
+                const float r = r2 * rsqrt_normal(r2), a = 1.0f - half_inv_h * r;
+                const float dot = (vi[0] - Wj.x) * d[0] + (vi[1] - Wj.y) * d[1] +
+                                  (D == 3 ? (vi[2] - Wj.z) * d[2] : 0.0f);
+                // (v_i - v~_ij).grad_i W = dW / r [(v_i - v_j).d / 2 + r (p_i - p_j) / ((rho_i + rho_j) c0)]
+                const float diff = 0.5f * dot + r * __fdividef(dp(Wj.w), (rhoi + rhoj) * P.c0);
+                rate += __fdividef(a * a * a * mdW, rhoj) * diff;
             }, none, none);
     }
     rate = group_sum<L>(rate);
@@ -225,7 +223,7 @@ __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, cons
             sS = ff_add(sS, W_ff_shape<D>(Pi, Li, Aq, s.L4[q], ox, oy, oz, g, P));
         };
         // the screen passes pairs up to 1.0001 (2 h)^2; W_ff_shape returns 0 beyond the support
-        fluid_pairs<D, L, CP, FORM, SETS, SETS == kAllSets>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, screen, list, stride, ts,
+        fluid_pairs<D, L, CP, FORM, SETS, SETS == kAllSets, false>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, screen, list, stride, ts,
                                 [&](int j) { return f.L4[j]; },
                                 [&](int, const float4 &Pj, const float4 &Lj, const float *, float, float ox, float oy,
                                     float oz) {

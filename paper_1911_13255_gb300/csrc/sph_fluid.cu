@@ -37,6 +37,8 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
         int cx, cy, cz;
         cell_xyz<D>(f.cell_of[i], In, cx, cy, cz);
         const float c0 = P.c0, eta2 = 2.0f * P.eta;
+        // dW / r = dWcF / h (1 - r / 2h)^3
+        const float half_inv_h = 0.5f * P.inv_hF, mdW = P.mF * (P.dWcF * P.inv_hF);
         // walls (v~ = a~ = 0) and solid particles at their start-of-step
         // positions with v~, a~
         auto wall_pair = [&](int a, float ox, float oy, float oz) {
@@ -69,21 +71,20 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
                                           float, float) {
                 // two particles at one FP32 position (a clumped pair): the
                 // direction is undefined and the pair's terms vanish with r
-                if (r2 == 0.0f) return;
+                if (!(r2 >= kMinNormal)) return;
                 const float rhoj = P.rho0 + Vj.w;
-                // one reciprocal square root for 1/r and r (r2 > 0 here)
-                const float invr = rsqrtf(r2), r = r2 * invr;
-                float dW = dW_F(r, P);
-                // U = v.e with e = -d / r (from i to j)
-                float UL = -(vi[0] * d[0] + vi[1] * d[1] + (D == 3 ? vi[2] * d[2] : 0.0f)) * invr;
-                float UR = -(Vj.x * d[0] + Vj.y * d[1] + (D == 3 ? Vj.z * d[2] : 0.0f)) * invr;
-                float rb = 0.5f * (rhoi + rhoj);
-                float beta = fminf(3.0f * fmaxf(UL - UR, 0.0f), c0);
-                float Ps = 0.5f * (pi + Pj.w) + 0.5f * rb * beta * (UL - UR);
-                float sc = __fdividef(P.mF, rhoj) * dW * invr;   // V_j dW / r
-                acc[0] += sc * (-2.0f * Ps * d[0] + eta2 * (vi[0] - Vj.x));
-                acc[1] += sc * (-2.0f * Ps * d[1] + eta2 * (vi[1] - Vj.y));
-                if (D == 3) acc[2] += sc * (-2.0f * Ps * d[2] + eta2 * (vi[2] - Vj.z));
+                const float invr = rsqrt_normal(r2);
+                const float a = 1.0f - half_inv_h * (r2 * invr);
+                // U_L - U_R = -(v_i - v_j).d / r (e = -d / r points from i to j)
+                const float dv[3] = {vi[0] - Vj.x, vi[1] - Vj.y, D == 3 ? vi[2] - Vj.z : 0.0f};
+                const float du = -(dv[0] * d[0] + dv[1] * d[1] + (D == 3 ? dv[2] * d[2] : 0.0f)) * invr;
+                const float beta = fminf(3.0f * fmaxf(du, 0.0f), c0);
+                // 2 P* = p_i + p_j + (rho_i + rho_j) / 2 beta (U_L - U_R)
+                const float P2 = (pi + Pj.w) + (0.5f * (rhoi + rhoj)) * (beta * du);
+                const float sc = __fdividef(a * a * a * mdW, rhoj);   // V_j dW / r
+                acc[0] += sc * (eta2 * dv[0] - P2 * d[0]);
+                acc[1] += sc * (eta2 * dv[1] - P2 * d[1]);
+                if (D == 3) acc[2] += sc * (eta2 * dv[2] - P2 * d[2]);
             }, wall_pair, solid_pair);
     }
     for (int k = 0; k < D; k++) {
@@ -107,8 +108,10 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
         f.W4[i] = make_float4(vn[0], vn[1], vn[2], Vi.w);
         if (SETS != kFluidOnly) f.B4[i] = make_float4(bnd[0], bnd[1], bnd[2], bnd[3]);
         cnt.vmax = sqrtf(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
-        float Vi_ = P.mF / rhoi;   // force = V_i * afs (same V_i as the solid side)
-        for (int k = 0; k < D; k++) cnt.mom[k] = (double)(Vi_ * afs[k]);
+        if (SETS == kAllSets) {
+            float Vi_ = P.mF / rhoi;   // force = V_i * afs (same V_i as the solid side)
+            for (int k = 0; k < D; k++) cnt.mom[k] = (double)(Vi_ * afs[k]);
+        }
     }
     flush_counts<D>(bt, b, act, cnt, true);
 }

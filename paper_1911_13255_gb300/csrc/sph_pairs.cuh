@@ -152,10 +152,18 @@ __device__ __forceinline__ void cell_offset(int code, const Grid &g, float &ox, 
 }
 
 // Cell offset of a neighbour-row entry: 2 bits per axis, (dx + 1) | (dy + 1)
-// << 2 | (dz + 1) << 4 (reach 1), decoded with shifts and masks.
+// << 2 | (dz + 1) << 4 (reach 1).  The bits go to the bottom of the mantissa of
+// 2^23, where a subtraction turns them into 1 - b, 4 (1 - b) or 16 (1 - b)
+// exactly (two full-rate instructions; a shift, a mask and an integer
+// conversion, which has an eighth of their rate, before).
 __device__ __forceinline__ uint32_t row_code(int code27)
 {
     return (uint32_t)(code27 % 3) | (uint32_t)((code27 / 3) % 3) << 2 | (uint32_t)(code27 / 9) << 4;
+}
+__device__ __forceinline__ float row_step(uint32_t e, int axis)
+{
+    const uint32_t bits = (e & (3u << (2 * axis))) | 0x4b000000u;
+    return (float)(8388608 + (1 << (2 * axis))) - __uint_as_float(bits);
 }
 __device__ __forceinline__ void row_offset(uint32_t e, const Grid &g, float &ox, float &oy, float &oz)
 {
@@ -164,12 +172,46 @@ __device__ __forceinline__ void row_offset(uint32_t e, const Grid &g, float &ox,
     oz = (float)(1 - (int)((e >> 4) & 3u)) * g.csf[2];
 }
 
+// Four entries of each of 4 neighbouring lanes (16 consecutive entries of a
+// row), transposed: value k of the 4 lanes then is entries 4 k .. 4 k + 3, whose
+// records mostly share lines.
+__device__ __forceinline__ uint4 transpose4(uint4 e, int lane, unsigned group)
+{
+    const bool odd = lane & 1, high = lane & 2;
+    uint32_t r0 = __shfl_xor_sync(group, odd ? e.x : e.y, 1), r1 = __shfl_xor_sync(group, odd ? e.z : e.w, 1);
+    if (odd) e.x = r0, e.z = r1;
+    else e.y = r0, e.w = r1;
+    r0 = __shfl_xor_sync(group, high ? e.x : e.z, 2);
+    r1 = __shfl_xor_sync(group, high ? e.y : e.w, 2);
+    if (high) e.x = r0, e.y = r1;
+    else e.z = r0, e.w = r1;
+    return e;
+}
+
 template <int D>
 __device__ __forceinline__ float rel_d(const float4 &Pi, const float4 &Pj, float ox, float oy, float oz, float d[3])
 {
     d[0] = (Pi.x - Pj.x) + ox;
     d[1] = (Pi.y - Pj.y) + oy;
     d[2] = D == 3 ? (Pi.z - Pj.z) + oz : 0.0f;
+    return d[0] * d[0] + d[1] * d[1] + (D == 3 ? d[2] * d[2] : 0.0f);
+}
+
+// the same for row entry e: (P_i - P_j) + o with o = step * edge, which one fused
+// multiply-add rounds like the sum (the product is exact)
+struct RowEdges {
+    float x, y, z;
+    __device__ __forceinline__ explicit RowEdges(const Grid &g)
+        : x(g.csf[0]), y(0.25f * g.csf[1]), z(0.0625f * g.csf[2])
+    {
+    }
+};
+template <int D>
+__device__ __forceinline__ float rel_row(const float4 &Pi, const float4 &Pj, uint32_t e, const RowEdges &c, float d[3])
+{
+    d[0] = __fmaf_rn(row_step(e, 0), c.x, Pi.x - Pj.x);
+    d[1] = __fmaf_rn(row_step(e, 1), c.y, Pi.y - Pj.y);
+    d[2] = D == 3 ? __fmaf_rn(row_step(e, 2), c.z, Pi.z - Pj.z) : 0.0f;
     return d[0] * d[0] + d[1] * d[1] + (D == 3 ? d[2] * d[2] : 0.0f);
 }
 
@@ -556,8 +598,9 @@ __device__ __forceinline__ unsigned fluid_pairs_rows(const Fluid &f, const Walls
 // visited only when the row says there are any; a row that overflowed takes
 // the cell form.  Pairs in a row are in support by construction: pair() gets
 // them without a test (the count of this lane's fluid pairs is returned).
-// OVER: the caller's targets include overflowed rows.
-template <int D, int L, int BND, bool OVER, typename Fetch, typename Pair, typename WP, typename SP>
+// OVER: the caller's targets include overflowed rows.  WIDE: row entries by
+// 16-byte loads.
+template <int D, int L, int BND, bool OVER, bool WIDE, typename Fetch, typename Pair, typename WP, typename SP>
 __device__ __forceinline__ unsigned fluid_pairs_list(const Fluid &f, const Walls &w, const Solid &s, const Grid &g,
                                                      int c0, int cx, int cy, int cz, int i, int lane,
                                                      const float4 &Pi, float rc2, Fetch &fetch, Pair &pair, WP &wp,
@@ -577,33 +620,57 @@ __device__ __forceinline__ unsigned fluid_pairs_list(const Fluid &f, const Walls
     }
     const int nF = (int)(cw & kListCountMask), nW = (int)((cw >> 11) & kListCountMask);
     const uint32_t *__restrict__ row = f.nbl + (size_t)i * f.list_cap;
-    // two entries per lane per round, both gathers issued before either pair
-    // is evaluated (the loop is bound by the latency of entry -> record
-    // chains); the pairs are summed in the same order as one at a time
-    int q = lane;
-    for (; q + L < nF; q += 2 * L) {
-        const uint32_t e0 = row[q], e1 = row[q + L];
+    // two records at a time, both gathers issued before either pair is evaluated
+    const RowEdges edge(g);
+    unsigned mine = 0;
+    auto two = [&](uint32_t e0, uint32_t e1) {
         const int j0 = (int)(e0 >> kCodeBits), j1 = (int)(e1 >> kCodeBits);
         const float4 P0 = f.P4[j0], P1 = f.P4[j1];
         const auto X0 = fetch(j0);
         const auto X1 = fetch(j1);
-        float ox, oy, oz, d[3];
+        float d[3], ox, oy, oz;
+        float r2 = rel_row<D>(Pi, P0, e0, edge, d);
         row_offset(e0, g, ox, oy, oz);
-        float r2 = rel_d<D>(Pi, P0, ox, oy, oz, d);
         pair(j0, P0, X0, d, r2, ox, oy, oz);
+        r2 = rel_row<D>(Pi, P1, e1, edge, d);
         row_offset(e1, g, ox, oy, oz);
-        r2 = rel_d<D>(Pi, P1, ox, oy, oz, d);
         pair(j1, P1, X1, d, r2, ox, oy, oz);
+        mine += 2;
+    };
+    int q = lane;
+    if constexpr (WIDE && L >= 4) {
+        // Whole blocks of 16 entries, 4 lanes a block, one 16-byte load per lane
+        // for four pairs, the next one under way meanwhile.  The loop is bound by
+        // the L1 lines its loads touch and by the latency of the entry -> record
+        // chain, whose first link comes from DRAM for a large problem (3-D duct,
+        // 375k particles, alone: continuity 139 -> 116 us, momentum 184 -> 168 us
+        // with the arithmetic of the pairs; one entry per load touches a line per
+        // target and load, 8 of the 32 lines of a warp's 32 pairs).  Not for the
+        // reinitialisation, which its arithmetic bounds: 107 -> 117 us per step.
+        const uint4 *__restrict__ row4 = (const uint4 *)row;
+        const unsigned group = 0xfu << (threadIdx.x & 28);
+        const int units = 4 * (nF >> 4);
+        uint4 next = make_uint4(0u, 0u, 0u, 0u);
+        if (lane < units) next = row4[lane];
+        for (int u = lane; u < units; u += L) {
+            const uint4 e = transpose4(next, lane, group);
+            if (u + L < units) next = row4[u + L];
+            two(e.x, e.y);
+            two(e.z, e.w);
+        }
+        q += 4 * units;
+    } else {
+        for (; q + L < nF; q += 2 * L) two(row[q], row[q + L]);
     }
-    if (q < nF) {
+    for (; q < nF; q += L) {
         const uint32_t e = row[q];
         const int j = (int)(e >> kCodeBits);
-        float ox, oy, oz;
-        row_offset(e, g, ox, oy, oz);
         const float4 Pj = f.P4[j];
-        float d[3];
-        const float r2 = rel_d<D>(Pi, Pj, ox, oy, oz, d);
+        float d[3], ox, oy, oz;
+        const float r2 = rel_row<D>(Pi, Pj, e, edge, d);
+        row_offset(e, g, ox, oy, oz);
         pair(j, Pj, fetch(j), d, r2, ox, oy, oz);
+        mine++;
     }
     if constexpr (BND != kFluidOnly) {
         const uint32_t *__restrict__ wrow = row + f.list_cap - 1;   // wall entries run from the back
@@ -621,7 +688,7 @@ __device__ __forceinline__ unsigned fluid_pairs_list(const Fluid &f, const Walls
                 });
         }
     }
-    return lane < nF ? (unsigned)((nF - lane + L - 1) / L) : 0u;
+    return mine;
 }
 
 // All neighbours of target i: fluid-fluid pairs through pair (their number
@@ -630,14 +697,14 @@ __device__ __forceinline__ unsigned fluid_pairs_list(const Fluid &f, const Walls
 // the cell form visits the fluid cells (from the staged tile when ts is set),
 // then the wall and solid entries cell by cell, over the 3^d cells (FORM 0)
 // or the 5^d cells of edge >= h_F (FORM 2).
-template <int D, int L, bool CP, int FORM, int BND, bool OVER, typename Fetch, typename Pair, typename WP, typename SP>
+template <int D, int L, bool CP, int FORM, int BND, bool OVER, bool WIDE = true, typename Fetch, typename Pair, typename WP, typename SP>
 __device__ __forceinline__ unsigned fluid_pairs(const Fluid &f, const Walls &w, const Solid &s, const Grid &g, int c0,
                                                 int cx, int cy, int cz, int i, int lane, const float4 &Pi, float rc2,
                                                 uint32_t *list, int stride, const TileSrc *ts, Fetch &&fetch,
                                                 Pair &&pair, WP &&wp, SP &&sp)
 {
     if constexpr (FORM == 3) {
-        return fluid_pairs_list<D, L, BND, OVER>(f, w, s, g, c0, cx, cy, cz, i, lane, Pi, rc2, fetch, pair, wp, sp);
+        return fluid_pairs_list<D, L, BND, OVER, WIDE>(f, w, s, g, c0, cx, cy, cz, i, lane, Pi, rc2, fetch, pair, wp, sp);
     } else if constexpr (FORM == 1) {
         return fluid_pairs_rows<D, L, CP, BND>(f, w, s, g, c0, cx, cy, cz, i, lane, Pi, rc2, list, stride, fetch, pair, wp,
                                           sp);
@@ -672,19 +739,43 @@ __device__ __forceinline__ double group_sum_d(double v)
 // p_i - p_j of Eq. eqeos without cancellation: with a = 1 + drho_i / rho0 and
 // b = 1 + drho_j / rho0, p_i - p_j = (rho0 c^2 / 7) (a^7 - b^7)
 //                                  = (rho0 c^2 / 7) (a - b) sum_k a^k b^(6-k)
-__device__ __forceinline__ float eos_dp(float drho_i, float drho_j, const Phys &P)
+// (the target's powers once per target)
+struct EosDiff {
+    float inv, drho, a1, a2, a3, a4, a5, a6, scale;
+    __device__ __forceinline__ EosDiff(float drho_i, const Phys &P)
+    {
+        inv = 1.0f / P.rho0;
+        drho = drho_i;
+        a1 = 1.0f + drho_i * inv;
+        a2 = a1 * a1;
+        a3 = a2 * a1;
+        a4 = a2 * a2;
+        a5 = a4 * a1;
+        a6 = a4 * a2;
+        scale = P.p_coef * inv;
+    }
+    __device__ __forceinline__ float operator()(float drho_j) const
+    {
+        const float b = 1.0f + drho_j * inv;
+        float s = a1 + b;
+        s = a2 + b * s;
+        s = a3 + b * s;
+        s = a4 + b * s;
+        s = a5 + b * s;
+        s = a6 + b * s;
+        return scale * (drho - drho_j) * s;
+    }
+};
+
+// 1/sqrt of a normal number (2 ulp; rsqrtf with its handling of subnormals,
+// which the pair loops send away first)
+__device__ __forceinline__ float rsqrt_normal(float x)
 {
-    float inv = 1.0f / P.rho0;
-    float a = 1.0f + drho_i * inv, b = 1.0f + drho_j * inv;
-    float s = a + b;
-    s = a * a + b * s;
-    s = a * a * a + b * s;
-    s = a * a * a * a + b * s;
-    float a2 = a * a;
-    s = a2 * a2 * a + b * s;
-    s = a2 * a2 * a2 + b * s;
-    return P.p_coef * ((drho_i - drho_j) * inv) * s;
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
+constexpr float kMinNormal = 1.17549435e-38f;
 
 // local cell coordinates of a global cell index (integer divisions are long
 // instruction sequences: one per axis beyond the first)
@@ -769,8 +860,11 @@ __device__ __forceinline__ void flush_counts(Batch bt, int b, bool valid, Counts
     if (warp_uniform(valid ? b : -1)) {
         unsigned ff = warp_sum_u(c.ff), fw = warp_sum_u(c.fw), fs = warp_sum_u(c.fs), sf = warp_sum_u(c.sf);
         float vm = warp_max(c.vmax);
+        // FP64 sums only where there are such pairs: the unit is slow enough
+        // for empty ones to take a third of the momentum loop's time
         double m[3] = {0.0, 0.0, 0.0};
-        for (int k = 0; k < D; k++) m[k] = warp_sum_d(c.mom[k]);
+        if (fluid_side ? fs : sf)
+            for (int k = 0; k < D; k++) m[k] = warp_sum_d(c.mom[k]);
         if ((threadIdx.x & 31) == 0 && valid) {
             Ctl *ctl = bt.ctl + b;
             if (ff) atomicAdd(&ctl->n_ff, (unsigned long long)ff);
