@@ -19,6 +19,8 @@
 // The deformation gradient is stored as H = F - I (FP32) so that small
 // strains keep their precision: E = (H + H^T + H^T H) / 2, ln J =
 // log1p(det(I + H) - 1), S = C^-1 (2 mu E + lambda ln J I).
+#include <algorithm>
+
 #include "sph_common.cuh"
 
 namespace sph {
@@ -1828,14 +1830,22 @@ static size_t window_smem(int dim, int slots, int own)
 }
 
 // Shape of the windowed kernel for a body of n particles: particles per CTA
-// and threads per CTA.  One CTA per SM at most; a small body is spread over
-// fewer CTAs of kWinMinOwn particles, since a CTA's phase costs a few L2
-// round trips however little it holds.
-void solid_window_shape(int dim, int n, int nsm, int *own, int *threads)
+// and threads per CTA.  At most one CTA per SM, and at least 32 particles each,
+// since a CTA's phase costs a few L2 round trips however little it holds.
+// Between these bounds, as many particles per CTA as let a sub-step take about
+// sub_us: a CTA's 512 threads of 128 registers leave its SM to nothing else, so
+// when the fluid loops are the longer branch the sub-steps should hide behind
+// them on few SMs.  A sub-step takes about 8 + 0.055 P us in 3-D, 4 + 0.02 P us in
+// 2-D (P particles per CTA).  3-D duct, 375k fluid and 8160 solid particles: step
+// 881 us with 152 CTAs, 806 with 76, 775 with 38, 820 with 24; 2-D gate of 6400
+// particles, the longer branch there: 188 us with 152, 186 with 100, 278 with 25.
+void solid_window_shape(int dim, int n, int nsm, double sub_us, int *own, int *threads)
 {
-    const int L = dim == 3 ? kWinL<3> : kWinL<2>, least = 32;
-    int P = (n + nsm - 1) / nsm;
-    if (P < least) P = least;
+    const int L = dim == 3 ? kWinL<3> : kWinL<2>;
+    const int least = std::max(32, (n + nsm - 1) / nsm);
+    const double fit = dim == 3 ? (sub_us - 8.0) / 0.055 : (sub_us - 4.0) / 0.02;
+    int P = (int)std::min(std::max(fit, (double)least), (double)kWinThreads);
+    P = std::max(std::min(P, n), least);
     int T = (P * L + 31) / 32 * 32;
     if (T > kWinThreads) T = kWinThreads;
     if (T < (P + 31) / 32 * 32) T = (P + 31) / 32 * 32;
