@@ -102,7 +102,7 @@ int launch_density(const Batch &bt, const Fluid &f, const Walls &w, const Solid 
 {
     if (f.n == 0) return 0;
     if (f.n >= kMaxPairTargets) return -7;
-    SPH_LAUNCH_PAIRS(k_density, f.n, 0, bt, f, w, s);
+    SPH_LAUNCH_PAIRS(k_density, f.n, 0, kAllBlocks, bt, f, w, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -221,19 +221,36 @@ struct WendlandPairs {
     }
 };
 
-template <int D, int L, bool CP, int FORM, int SETS>
-__device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int i,
-                                                 bool act_, int lane, uint32_t *list, int stride, const TileSrc *ts)
+// The shape sums of one target over the fluid, the walls and the solid.
+struct ShapeSums {
+    ff f, w, s;
+};
+
+template <int L>
+__device__ __forceinline__ ff group_sum_ff(ff v)
 {
-    const int b = act_ ? f.inst[i] : 0;
-    // the L lanes of a particle share its instance, so this is group-uniform
-    const bool act = act_ && bt.ctl[b].reinit && (SETS == kAllSets || !(f.nbc[i] & (kListSolid | kListOver)));
-    const Inst &In = bt.I[b];
-    const Grid &g = In.g;
-    const Phys &P = In.P;
-    const float screen = P.rc2F * 1.0001f;
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, v.hi, o), l = __shfl_xor_sync(0xffffffffu, v.lo, o);
+        const ff t = ff_two_sum(v.hi, h);
+        v.hi = t.hi;
+        v.lo = __fadd_rn(__fadd_rn(v.lo, l), t.lo);
+    }
+    return v;
+}
+
+// (over its L lanes, in every lane)
+template <int D, int L, bool CP, int FORM, int SETS>
+__device__ __forceinline__ ShapeSums reinit_pairs(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s,
+                                                  int i, bool act, int lane, uint32_t *list, int stride,
+                                                  const TileSrc *ts)
+{
     ff sF = {0.0f, 0.0f}, sW = {0.0f, 0.0f}, sS = {0.0f, 0.0f};
     if (act) {
+        const Inst &In = bt.I[f.inst[i]];
+        const Grid &g = In.g;
+        const Phys &P = In.P;
+        const float screen = P.rc2F * 1.0001f;
         const float4 Pi = f.P4[i], Li = f.L4[i];
         const WendlandPairs<D> shape(g, P, Pi, Li);
         int cx, cy, cz;
@@ -250,17 +267,21 @@ __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, cons
             if (rel_d<D>(Pi, Aq, ox, oy, oz, d) >= screen) return;
             shape.add(sS, Aq, s.L4[q], ox, oy, oz);
         };
-        fluid_pairs<D, L, CP, FORM, SETS, SETS == kAllSets, false>(f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, screen, list, stride, ts,
-                                [&](int j) { return f.L4[j]; },
-                                [&](int, const float4 &Pj, const float4 &Lj, const float *, float, float ox, float oy,
-                                    float oz) {
+        fluid_pairs<D, L, CP, FORM, SETS, SETS == kAllSets, false>(
+            f, w, s, g, In.c0, cx, cy, cz, i, lane, Pi, screen, list, stride, ts, [&](int j) { return f.L4[j]; },
+            [&](int, const float4 &Pj, const float4 &Lj, const float *, float, float ox, float oy, float oz) {
                 shape.add(sF, Pj, Lj, ox, oy, oz);
-            }, wall_pair, solid_pair);
+            },
+            wall_pair, solid_pair);
     }
-    const double dF = group_sum_d<L>((double)sF.hi + (double)sF.lo);
-    const double dW = group_sum_d<L>((double)sW.hi + (double)sW.lo);
-    const double dS = group_sum_d<L>((double)sS.hi + (double)sS.lo);
-    if (!act || lane != 0) return;
+    return {group_sum_ff<L>(sF), group_sum_ff<L>(sW), SETS == kAllSets ? group_sum_ff<L>(sS) : sS};
+}
+
+__device__ __forceinline__ void reinit_finish(const Batch &bt, const Fluid &f, int i, const ShapeSums &v)
+{
+    const Phys &P = bt.I[f.inst[i]].P;
+    const double dF = (double)v.f.hi + (double)v.f.lo, dW = (double)v.w.hi + (double)v.w.lo,
+                 dS = (double)v.s.hi + (double)v.s.lo;
     double sigma = P.alphaF_d * (1.0 + dF + P.VW_VF_d * dW + P.VS_VF_d * dS);
     double dr = P.rho0_d * ((sigma - P.sigma0_d) / P.sigma0_d);
     if (P.free_surface && dr < 0.0) dr = 0.0;
@@ -272,33 +293,58 @@ __device__ __forceinline__ void reinit_one(const Batch &bt, const Fluid &f, cons
 
 // Row form: the targets near solid particles and those of overflowed rows take
 // a warp each, in the first blocks (as in k_momentum; the walls, whose pairs
-// cost no more than the fluid's here, stay with the rest).
+// cost no more than the fluid's here, stay with the rest).  The FP64 end of a
+// target's sums runs in whole warps (FP64 takes as long for 4 active lanes as
+// for 32; 32 flow channels 57 -> 41 us of a step).  On most steps no instance is due: a grid of some 30 waves strides over the targets, so
+// that such a step costs a launch and not one block per 32 targets (3-D duct,
+// 3.0M particles: 121 us, now 22).
+constexpr int kReinitBlocks = 152 * 128;
+
 template <int D, int L, bool CP, bool TILE, int FORM>
 __global__ void __launch_bounds__(kMaxBlock, D == 2 && FORM != 1 ? 5 : (D == 3 && FORM == 1 ? 3 : 4)) k_reinit(Batch bt, Fluid f, Walls w, Solid s)
 {
     pdl_enter();
     if (step_failed(bt)) return;   // the step's cell starts are not valid
+    if (bt.B == 1 && !bt.ctl[0].reinit) return;
     extern __shared__ __align__(16) uint8_t s_dyn[];
     uint32_t *const list = (uint32_t *)s_dyn + threadIdx.x;
-    const int stride = blockDim.x;
-    if constexpr (FORM == 3) {
-        const int nn = part_blocks(f.n, kPartNear, blockDim.x), k = blockIdx.x;
-        if (k < nn) {
-            part_loop<32>(f, kPartNear, k, nn, [&](int i, bool act, int lane) {
-                reinit_one<D, 32, CP, FORM, kAllSets>(bt, f, w, s, i, act, lane, nullptr, 0, nullptr);
+    const int stride = blockDim.x, lane = (int)threadIdx.x % L;
+    constexpr int SETS = FORM == 3 ? kFluidWall : kAllSets;
+    // is this a reinitialisation step of target i's instance?
+    auto due = [&](int i) { return i < f.n && bt.ctl[f.inst[i]].reinit; };
+    if constexpr (!TILE) {
+        const int nn = FORM == 3 ? part_blocks(f.n, kPartNear, blockDim.x) : 0;
+        if ((int)blockIdx.x < nn) {
+            part_loop<32>(f, kPartNear, blockIdx.x, nn, [&](int i, bool act, int l) {
+                const bool go = act && due(i);
+                const ShapeSums v = reinit_pairs<D, 32, CP, FORM, kAllSets>(bt, f, w, s, i, go, l, nullptr, 0, nullptr);
+                if (go && l == 0) reinit_finish(bt, f, i, v);
             });
-        } else {
-            const int t = (k - nn) * blockDim.x + threadIdx.x;
-            reinit_one<D, L, CP, FORM, kFluidWall>(bt, f, w, s, t / L, t / L < f.n, t % L, nullptr, 0, nullptr);
+            return;
         }
-    } else if constexpr (!TILE) {
-        const int t = blockIdx.x * blockDim.x + threadIdx.x;
-        reinit_one<D, L, CP, FORM, kAllSets>(bt, f, w, s, t / L, t / L < f.n, t % L, list, stride, nullptr);
+        __shared__ ShapeSums s_sums[kMaxBlock / L];
+        auto mine = [&](int i) {
+            return due(i) && (FORM != 3 || !(f.nbc[i] & (kListSolid | kListOver)));
+        };
+        const int per = blockDim.x / L, k = (int)threadIdx.x / L, step = ((int)gridDim.x - nn) * per;
+        for (int i0 = ((int)blockIdx.x - nn) * per; i0 < f.n; i0 += step) {
+            const bool act = mine(i0 + k);
+            if (!__syncthreads_or(act)) continue;   // no instance of these targets is due
+            const ShapeSums v =
+                reinit_pairs<D, L, CP, FORM, SETS>(bt, f, w, s, i0 + k, act, lane, list, stride, nullptr);
+            if (lane == 0) s_sums[k] = v;
+            __syncthreads();
+            if ((int)threadIdx.x < per && mine(i0 + threadIdx.x))
+                reinit_finish(bt, f, i0 + threadIdx.x, s_sums[threadIdx.x]);
+        }
     } else {
         if (!bt.ctl[f.tiles[blockIdx.x].x].reinit) return;   // not a reinitialisation step of this instance
         tile_loop<D, L>(bt, f, f.L4, s_dyn + (CP ? (size_t)kListBytes * blockDim.x : 0),
                         [&](int i, bool act, const TileSrc *ts) {
-                            reinit_one<D, L, CP, FORM, kAllSets>(bt, f, w, s, i, act, (int)threadIdx.x % L, list, stride, ts);
+                            const bool go = act && due(i);
+                            const ShapeSums v =
+                                reinit_pairs<D, L, CP, FORM, kAllSets>(bt, f, w, s, i, go, lane, list, stride, ts);
+                            if (go && lane == 0) reinit_finish(bt, f, i, v);
                         });
     }
 }
@@ -307,7 +353,7 @@ int launch_reinit(const Batch &bt, const Fluid &f, const Walls &w, const Solid &
 {
     if (f.n == 0) return 0;
     if (f.n >= kMaxPairTargets) return -7;
-    SPH_LAUNCH_PAIRS(k_reinit, f.n, f.list ? part_blocks(f.n, kPartNear, f.block) : 0, bt, f, w, s);
+    SPH_LAUNCH_PAIRS(k_reinit, f.n, f.list ? part_blocks(f.n, kPartNear, f.block) : 0, kReinitBlocks, bt, f, w, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

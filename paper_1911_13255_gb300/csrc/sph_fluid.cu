@@ -170,7 +170,7 @@ int launch_momentum(const Batch &bt, const Fluid &f, const Walls &w, const Solid
     if (f.n == 0) return 0;
     if (f.n >= kMaxPairTargets) return -7;
     const int parts = f.list ? part_blocks(f.n, kPartNear, f.block) + part_blocks(f.n, kPartWall, f.block) : 0;
-    SPH_LAUNCH_PAIRS(k_momentum, f.n, parts, bt, f, w, s);
+    SPH_LAUNCH_PAIRS(k_momentum, f.n, parts, kAllBlocks, bt, f, w, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

@@ -942,13 +942,17 @@ static void allow_smem(K kern, size_t bytes)
     if (bytes > 32 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-#define SPH_LAUNCH_PAIRS(KERN, n, extra, ...)                                                      \
+// (at most `most` blocks over the targets, plus `extra`)
+constexpr int kAllBlocks = 0x7fffffff;
+
+#define SPH_LAUNCH_PAIRS(KERN, n, extra, most, ...)                                                      \
     do {                                                                                      \
         const size_t sm_ = f.list ? 0 : (f.compact ? (size_t)kListBytes * f.block : 0) +     \
                            (f.tile ? (size_t)f.tile_cap * 32 : 0);                            \
         auto go_ = [&](auto Dc, auto Lc) {                                                    \
             constexpr int D_ = decltype(Dc)::value, L_ = decltype(Lc)::value;                \
-            const int nb_ = f.tile ? f.ntiles : grid_blocks(n, L_, f.block) + (extra);        \
+            const int all_ = grid_blocks(n, L_, f.block);                                     \
+            const int nb_ = f.tile ? f.ntiles : (all_ < (most) ? all_ : (most)) + (extra);    \
             if (nb_ == 0) return;                                                             \
             auto run_ = [&](auto kern) {                                                      \
                 allow_smem(kern, sm_);                                                        \
