@@ -16,7 +16,15 @@
 //     groups, +32 B per K step inside the swizzle atom) and commits them to the
 //     stage's "empty" mbarrier; after the last chunk it commits to "done";
 //   - all four warps wait for "done", read the accumulator with tcgen05.ld
-//     (warp w owns TMEM lanes 32w..32w+31 = tile rows), add the bias and store.
+//     (warp w owns TMEM lanes 32w..32w+31 = tile rows), turn 32 x 32 blocks
+//     through shared memory (the ring is free by then), add the bias and store
+//     128 bytes of a row per 8 lanes.
+// A chunk of a 128 x 256 tile costs shared memory 48 KB of TMA writes and 48 KB
+// of operand reads against 512 cycles of MMA, which bounds large products:
+// 4096 x 4096 x 4096 takes 124 us (1.11 PFLOP/s; 312 us with the idle lanes of
+// warps 0 and 1 spinning next to their lane 0 and a row of 16-byte stores per
+// lane), 16384 x 256 x 4096 48 us (85).  Sharing B in clusters of 2 or 4 by
+// multicast, prefetching A into L2 and 256-byte L2 promotion change neither.
 // Every wait is bounded; a timeout sets a status bit, skips the epilogue and
 // still frees the tensor memory.
 #include <cuda.h>   // CUtensorMap and its enums; the encoder comes from the CUDA driver library at run time
@@ -79,12 +87,13 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr)
 }
 
 constexpr int kStages = 4;
+constexpr int kEpiLd = 36;   // floats per row of a warp's 32 x 32 epilogue block (16-byte rows, 8 lanes without conflicts)
 
 template <int NT>
 __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant__ CUtensorMap tmA,
                                                           const __grid_constant__ CUtensorMap tmB,
                                                           const float *__restrict__ bias, float *__restrict__ C,
-                                                          int M, int N, int K, int kper)
+                                                          int M, int N, int K, int kper, int stages)
 {
     // split K: slice blockIdx.z covers chunks [z kper, (z + 1) kper) and
     // writes its partial tile to C + z M N (the caller reduces the slices)
@@ -100,7 +109,6 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant_
     const int m0 = blockIdx.x * 128, n0 = blockIdx.y * NT;
     const int kc0 = blockIdx.z * kper;
     const int nk = min(K / kKChunk - kc0, kper);
-
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(kCols)
@@ -123,15 +131,11 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant_
     bool ok = true;
     if (warp == 0 && lane == 0) {
         // producer
-        uint32_t ph[kStages] = {0u, 0u, 0u, 0u};
-        for (int kc = 0; kc < nk; kc++) {
-            const int s = kc % kStages;
-            if (kc >= kStages) {
-                if (!mbar_wait(smem_u32(&empty[s]), ph[s])) {
-                    ok = false;
-                    break;
-                }
-                ph[s] ^= 1u;
+        uint32_t ph = 1u;   // of the ring's previous round; the first finds every stage empty
+        for (int kc = 0, s = 0; kc < nk; kc++) {
+            if (!mbar_wait(smem_u32(&empty[s]), ph)) {
+                ok = false;
+                break;
             }
             const uint32_t a_s = base + s * kStage, b_s = a_s + kAStage, fb = smem_u32(&full[s]);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(kStage) : "memory");
@@ -145,17 +149,16 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant_
                 "[%4];" ::"r"(b_s),
                 "l"(reinterpret_cast<uint64_t>(&tmB)), "r"((kc0 + kc) * kKChunk), "r"(n0), "r"(fb)
                 : "memory");
+            if (++s == stages) s = 0, ph ^= 1u;
         }
     } else if (warp == 1 && lane == 0) {
         // MMA issuer
-        uint32_t ph[kStages] = {0u, 0u, 0u, 0u};
-        for (int kc = 0; kc < nk; kc++) {
-            const int s = kc % kStages;
-            if (!mbar_wait(smem_u32(&full[s]), ph[s])) {
+        uint32_t ph = 0u;
+        for (int kc = 0, s = 0; kc < nk; kc++) {
+            if (!mbar_wait(smem_u32(&full[s]), ph)) {
                 ok = false;
                 break;
             }
-            ph[s] ^= 1u;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t a0 = base + s * kStage, b0 = a0 + kAStage;
 #pragma unroll
@@ -173,43 +176,60 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant_
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              smem_u32(&empty[s]))
                          : "memory");
+            if (++s == stages) s = 0, ph ^= 1u;
         }
         // covers every MMA issued before it (arrives at once if there is none)
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                          smem_u32(&done))
                      : "memory");
     }
+    // the other lanes of warps 0 and 1 stay out of the wait below while lane 0
+    // works: spinning there, they share the warp's issue slot with it
+    __syncwarp();
     if (!mbar_wait(smem_u32(&done), 0u)) ok = false;
     ok = __syncthreads_and(ok);
     if (!ok && tid == 0) atomicOr(&g_tc_status, 1u);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
-        const int row = m0 + warp * 32 + lane;
+        constexpr int CW = NT < 32 ? NT : 32;   // columns per block
+        constexpr int kLn = CW / 4, kRw = 32 / kLn;   // lanes per row, rows per store
+        float *blk = reinterpret_cast<float *>(dsm + (base - smem_u32(dsm))) + warp * (32 * kEpiLd);
+        const int cc = 4 * (lane % kLn), rr = lane / kLn;
 #pragma unroll 1
-        for (int c = 0; c < NT; c += 16) {
-            uint32_t v[16];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-                "%13, %14, %15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15])
-                : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            float4 *out = (float4 *)(C + (size_t)row * N + n0 + c);
+        for (int c = 0; c < NT; c += CW) {
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                float4 o = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                       __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-                if (bias) {
-                    o.x += bias[n0 + c + 4 * j];
-                    o.y += bias[n0 + c + 4 * j + 1];
-                    o.z += bias[n0 + c + 4 * j + 2];
-                    o.w += bias[n0 + c + 4 * j + 3];
-                }
-                out[j] = o;
+            for (int h = 0; h < CW; h += 16) {
+                uint32_t v[16];
+                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c + h);
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                    "%13, %14, %15}, [%16];"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+                      "=r"(v[15])
+                    : "r"(taddr));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    *reinterpret_cast<uint4 *>(blk + lane * kEpiLd + h + 4 * j) =
+                        make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
+            __syncwarp();
+            float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (bias) bv = make_float4(bias[n0 + c + cc], bias[n0 + c + cc + 1], bias[n0 + c + cc + 2],
+                                       bias[n0 + c + cc + 3]);
+#pragma unroll
+            for (int k = 0; k < 32; k += kRw) {
+                float4 o = *reinterpret_cast<const float4 *>(blk + (k + rr) * kEpiLd + cc);
+                if (bias) {
+                    o.x += bv.x;
+                    o.y += bv.y;
+                    o.z += bv.z;
+                    o.w += bv.w;
+                }
+                *reinterpret_cast<float4 *>(C + (size_t)(m0 + warp * 32 + k + rr) * N + n0 + c + cc) = o;
+            }
+            __syncwarp();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -255,13 +275,16 @@ int make_map(CUtensorMap *m, const void *ptr, long long rows, long long cols, in
     return r == CUDA_SUCCESS ? 0 : -1;
 }
 
-// C = bias + sum of the S partial tiles, in slice order (deterministic)
+// C = bias + sum of the S partial tiles, in slice order (deterministic); eight
+// slices' loads in flight.  One value per thread: four would leave most SMs
+// without work (128 x 512 values of 34 slices: 6 us, 10 with four per thread).
 __global__ void k_splitk_sum(const float *__restrict__ ws, int S, long long MN, int N, const float *__restrict__ bias,
                              float *__restrict__ C)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MN) return;
     float v = bias ? bias[i % N] : 0.0f;
+#pragma unroll 8
     for (int z = 0; z < S; z++) v += ws[(size_t)z * MN + i];
     C[i] = v;
 }
@@ -275,10 +298,9 @@ int launch_tile(const uint16_t *A, const uint16_t *B, const float *bias, float *
                 cudaStream_t st)
 {
     constexpr int kStage = kAStage + NT * kKChunk * 2;
-    const int smem = kStages * kStage + 1024;
     static bool attr_set = false;
     if (!attr_set) {
-        if (cudaFuncSetAttribute(k_gemm_bf16<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+        if (cudaFuncSetAttribute(k_gemm_bf16<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * kStage + 1024) != cudaSuccess)
             return -3;
         attr_set = true;
     }
@@ -305,11 +327,13 @@ int launch_tile(const uint16_t *A, const uint16_t *B, const float *bias, float *
     }
     const int kper = (nk + S - 1) / S;
     S = (nk + kper - 1) / kper;
-    dim3 grid(M / 128, N / NT, S);
-    if (S == 1) {
-        k_gemm_bf16<NT><<<grid, kTcThreads, smem, st>>>(ta, tb, bias, C, M, N, K, kper);
-    } else {
-        k_gemm_bf16<NT><<<grid, kTcThreads, smem, st>>>(ta, tb, nullptr, g_ws, M, N, K, kper);
+    // a ring no longer than the K loop: short ones leave room for a second CTA on
+    // the SM (19072 x 512 x 128: 12.3 -> 11.0 us)
+    const int stages = std::min(kStages, kper), smem = stages * kStage + 1024;
+    const dim3 grid(M / 128, N / NT, S);
+    k_gemm_bf16<NT><<<grid, kTcThreads, smem, st>>>(ta, tb, S == 1 ? bias : nullptr, S == 1 ? C : g_ws, M, N, K, kper,
+                                                    stages);
+    if (S > 1) {
         const long long MN = (long long)M * N;
         k_splitk_sum<<<(unsigned)((MN + 255) / 256), 256, 0, st>>>(g_ws, S, MN, N, bias, C);
     }
