@@ -14,6 +14,7 @@
 // graph R times (block diagonal) so that R samples form one batch.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -65,51 +66,96 @@ __device__ __forceinline__ float dsilu_f(float y)
     return s + y * s * (1.0f - s);
 }
 
-// dst[r, c] = bf16(src[r, c]) for r < rows, c < cols (ld = row strides)
-__global__ void k_to_bf16(const float *__restrict__ src, int ld_src, int rows, int cols, bf16 *__restrict__ dst,
-                          int ld_dst)
+// four values rounded to bfloat16, as 8 bytes
+__device__ __forceinline__ uint2 pack4(float4 v)
 {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long long)rows * cols) return;
-    const int r = (int)(t / cols), c = (int)(t % cols);
-    dst[(size_t)r * ld_dst + c] = __float2bfloat16_rn(src[(size_t)r * ld_src + c]);
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
 }
 
-// mode 0: h = silu(y); mode 1: h += silu(y)
-__global__ void k_act(const float *__restrict__ y, float *__restrict__ h, long long n, int mode)
+// dst = bf16(src), 4 n4 values
+__global__ void k_to_bf16(const float4 *__restrict__ src, long long n4, uint2 *__restrict__ dst)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const float s = silu_f(y[t]);
-    h[t] = mode ? h[t] + s : s;
+    if (t < n4) dst[t] = pack4(src[t]);
 }
 
-// z row a = [bf16(h_a), bf16(m0_a), bf16(m1_a), ...]; one block (128
-// threads = channels) per real node; node a = r n + a0 uses the base graph
-// row a0 with neighbours r n + idx.
-template <int D>
-__global__ void __launch_bounds__(kC) k_aggregate(const float *__restrict__ h, bf16 *__restrict__ z, int n,
-                                                  const int *__restrict__ ptr, const int *__restrict__ idx,
-                                                  const float *__restrict__ w, const float *__restrict__ g)
+// mode 0: h = silu(y); mode 1: h += silu(y) (4 n4 values)
+__global__ void k_act(const float4 *__restrict__ y, float4 *__restrict__ h, long long n4, int mode)
 {
-    constexpr int zd = kC * (2 + D);
-    const int a = blockIdx.x, c = threadIdx.x;
-    const int r = a / n, a0 = a - r * n, off = r * n;
-    const float ha = h[(size_t)a * kC + c];
-    float m0 = 0.f, m[D];
-#pragma unroll
-    for (int k = 0; k < D; k++) m[k] = 0.f;
-    for (int q = ptr[a0]; q < ptr[a0 + 1]; q++) {
-        const float d = h[(size_t)(off + idx[q]) * kC + c] - ha;
-        m0 += w[q] * d;
-#pragma unroll
-        for (int k = 0; k < D; k++) m[k] += g[(size_t)q * D + k] * d;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n4) return;
+    const float4 v = y[t];
+    float4 s = make_float4(silu_f(v.x), silu_f(v.y), silu_f(v.z), silu_f(v.w));
+    if (mode) {
+        const float4 o = h[t];
+        s = make_float4(o.x + s.x, o.y + s.y, o.z + s.z, o.w + s.w);
     }
-    bf16 *zr = z + (size_t)a * zd;
-    zr[c] = __float2bfloat16_rn(ha);
-    zr[kC + c] = __float2bfloat16_rn(m0);
+    h[t] = s;
+}
+
+// The graph sums.  A warp takes a node, 4 channels per lane (16-byte loads of the
+// neighbours' rows, kNodeU of them in flight), and a block kNodes consecutive
+// nodes, whose neighbours are mostly the same rows: they come from L1.  One
+// block of 128 one-channel threads per node, as this was, read every row from
+// L2 and kept one load in flight (19 072 nodes of 20 neighbours, 2-D: sums 37 -> 20 us,
+// adjoint 51 -> 28 us).
+// Every channel's sum runs over the row's entries in order.
+constexpr int kNodes = 8, kNodeU = 4;
+
+__device__ __forceinline__ float4 sub4(float4 a, float4 b)
+{
+    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b)
+{
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+__device__ __forceinline__ void axpy4(float4 &m, float w, float4 d)
+{
+    m.x += w * d.x;
+    m.y += w * d.y;
+    m.z += w * d.z;
+    m.w += w * d.w;
+}
+
+// z row a = [bf16(h_a), bf16(m0_a), bf16(m1_a), ...]; node a = r n + a0 uses the
+// base graph row a0 with neighbours r n + idx.
+template <int D>
+__global__ void __launch_bounds__(32 * kNodes) k_aggregate(const float4 *__restrict__ h, uint2 *__restrict__ z, int n,
+                                                           int nn, const int *__restrict__ ptr,
+                                                           const int *__restrict__ idx, const float *__restrict__ w,
+                                                           const float *__restrict__ g)
+{
+    constexpr int C4 = kC / 4;
+    const int a = blockIdx.x * kNodes + (int)(threadIdx.x >> 5), c = threadIdx.x & 31;
+    if (a >= nn) return;
+    const int r = a / n, a0 = a - r * n, off = r * n;
+    const float4 ha = h[(size_t)a * C4 + c], zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 m0 = zero, m[D];
 #pragma unroll
-    for (int k = 0; k < D; k++) zr[(2 + k) * kC + c] = __float2bfloat16_rn(m[k]);
+    for (int k = 0; k < D; k++) m[k] = zero;
+    const int q1 = ptr[a0 + 1];
+    int q = ptr[a0];
+    auto entry = [&](int e, float4 hb) {
+        const float4 d = sub4(hb, ha);
+        axpy4(m0, w[e], d);
+#pragma unroll
+        for (int k = 0; k < D; k++) axpy4(m[k], g[(size_t)e * D + k], d);
+    };
+    for (; q + kNodeU <= q1; q += kNodeU) {
+        float4 hb[kNodeU];
+#pragma unroll
+        for (int u = 0; u < kNodeU; u++) hb[u] = h[(size_t)(off + idx[q + u]) * C4 + c];
+#pragma unroll
+        for (int u = 0; u < kNodeU; u++) entry(q + u, hb[u]);
+    }
+    for (; q < q1; q++) entry(q, h[(size_t)(off + idx[q]) * C4 + c]);
+    uint2 *zr = z + (size_t)a * C4 * (2 + D) + c;
+    zr[0] = pack4(ha);
+    zr[C4] = pack4(m0);
+#pragma unroll
+    for (int k = 0; k < D; k++) zr[(2 + k) * C4] = pack4(m[k]);
 }
 
 // Adjoint of the graph sums, for a symmetric neighbour relation with w
@@ -117,60 +163,112 @@ __global__ void __launch_bounds__(kC) k_aggregate(const float *__restrict__ h, b
 //   dh_b += dz_b[0:128] + sum_k sum_{a in N(b)} (s_k c^k_ba dm_k,a - c^k_ba dm_k,b)
 // with s_0 = +1 (w) and s_k = -1 (g).
 template <int D>
-__global__ void __launch_bounds__(kC) k_agg_adjoint(const float *__restrict__ dz, float *__restrict__ dh, int n,
-                                                    const int *__restrict__ ptr, const int *__restrict__ idx,
-                                                    const float *__restrict__ w, const float *__restrict__ g)
+__global__ void __launch_bounds__(32 * kNodes) k_agg_adjoint(const float4 *__restrict__ dz, float4 *__restrict__ dh,
+                                                             int n, int nn, const int *__restrict__ ptr,
+                                                             const int *__restrict__ idx, const float *__restrict__ w,
+                                                             const float *__restrict__ g)
 {
-    constexpr int zd = kC * (2 + D);
-    const int b = blockIdx.x, c = threadIdx.x;
+    constexpr int C4 = kC / 4, Z4 = C4 * (2 + D), U = 2;
+    const int b = blockIdx.x * kNodes + (int)(threadIdx.x >> 5), c = threadIdx.x & 31;
+    if (b >= nn) return;
     const int r = b / n, b0 = b - r * n, off = r * n;
-    const float *dzb = dz + (size_t)b * zd;
-    float acc = dzb[c];
-    float own[1 + D];
+    const float4 *dzb = dz + (size_t)b * Z4 + c;
+    float4 acc = dzb[0], own[1 + D];
 #pragma unroll
-    for (int k = 0; k <= D; k++) own[k] = dzb[(1 + k) * kC + c];
-    for (int q = ptr[b0]; q < ptr[b0 + 1]; q++) {
-        const float *dza = dz + (size_t)(off + idx[q]) * zd;
-        const float c0 = w[q];
-        acc += c0 * (dza[kC + c] - own[0]);
+    for (int k = 0; k <= D; k++) own[k] = dzb[(1 + k) * C4];
+    const int q1 = ptr[b0 + 1];
+    int q = ptr[b0];
+    auto load = [&](int e, float4 *v) {
+        const float4 *dza = dz + (size_t)(off + idx[e]) * Z4 + c;
 #pragma unroll
-        for (int k = 0; k < D; k++) {
-            const float ck = g[(size_t)q * D + k];
-            acc -= ck * (dza[(2 + k) * kC + c] + own[1 + k]);
+        for (int k = 0; k <= D; k++) v[k] = dza[(1 + k) * C4];
+    };
+    auto entry = [&](int e, const float4 *v) {
+        axpy4(acc, w[e], sub4(v[0], own[0]));
+#pragma unroll
+        for (int k = 0; k < D; k++) axpy4(acc, -g[(size_t)e * D + k], add4(v[1 + k], own[1 + k]));
+    };
+    for (; q + U <= q1; q += U) {
+        float4 v[U][1 + D];
+#pragma unroll
+        for (int u = 0; u < U; u++) load(q + u, v[u]);
+#pragma unroll
+        for (int u = 0; u < U; u++) entry(q + u, v[u]);
+    }
+    for (; q < q1; q++) {
+        float4 v[1 + D];
+        load(q, v);
+        entry(q, v);
+    }
+    float4 *o = dh + (size_t)b * C4 + c;
+    *o = add4(*o, acc);
+}
+
+// dy = dh * silu'(y) for the real rows, in bf16 (rows x 128), its transpose
+// (128 x np, read by the weight-gradient product) and db += column sums (FP32).
+// A block of 8 warps strides over tiles of 32 rows, a warp a row at a time, 4
+// channels per lane: 2 blocks per SM, so that the column sums end in few atomics
+// on the same 128 words (one block per tile: 18 us on 19 072 rows; now 10.6,
+// with the transpose that took 8 us of its own).
+__global__ void __launch_bounds__(256) k_dsilu(const float4 *__restrict__ dh, const float4 *__restrict__ y, int rows,
+                                               int np, uint2 *__restrict__ dy, bf16 *__restrict__ dyT,
+                                               float *__restrict__ db)
+{
+    constexpr int C4 = kC / 4;
+    __shared__ __align__(16) float s_sum[8][kC];
+    __shared__ __align__(8) bf16 s_dy[32][kC + 4];
+    const int c = threadIdx.x & 31, wr = threadIdx.x >> 5;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r0 = blockIdx.x * 32; r0 < np; r0 += gridDim.x * 32) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int rr = wr + 8 * k, r = r0 + rr;
+            uint2 q = make_uint2(0u, 0u);
+            if (r < rows) {
+                const float4 g = dh[(size_t)r * C4 + c], v = y[(size_t)r * C4 + c];
+                const float4 d = make_float4(g.x * dsilu_f(v.x), g.y * dsilu_f(v.y), g.z * dsilu_f(v.z),
+                                             g.w * dsilu_f(v.w));
+                q = pack4(d);
+                dy[(size_t)r * C4 + c] = q;
+                s = add4(s, d);
+            }
+            *reinterpret_cast<uint2 *>(&s_dy[rr][4 * c]) = q;
         }
+        __syncthreads();
+        // columns of the tile: 32 rows of one channel are 64 bytes of dyT (zeros past the last row)
+        for (int ch = wr; ch < kC; ch += 8) dyT[(size_t)ch * np + r0 + c] = s_dy[c][ch];
+        __syncthreads();
     }
-    dh[(size_t)b * kC + c] += acc;
+    *reinterpret_cast<float4 *>(&s_sum[wr][4 * c]) = s;
+    __syncthreads();
+    if (threadIdx.x < kC) {
+        float v = 0.f;
+        for (int k = 0; k < 8; k++) v += s_sum[k][threadIdx.x];
+        atomicAdd(&db[threadIdx.x], v);
+    }
 }
 
-// dy = dh * silu'(y) for the real rows; bf16 copy; db += column sums (FP32)
-__global__ void __launch_bounds__(kC) k_dsilu(const float *__restrict__ dh, const float *__restrict__ y, int rows,
-                                              bf16 *__restrict__ dy, float *__restrict__ db)
+// 64 x 64 tiled transpose: dst (cols x rows) = src (rows x cols)^T, rows and
+// cols multiples of 64; 16-byte loads and stores (2-byte ones in tiles of 32
+// moved 39 MB in 24 us; now 8.5)
+__global__ void __launch_bounds__(256) k_transpose(const bf16 *__restrict__ src, int rows, int cols,
+                                                   bf16 *__restrict__ dst)
 {
-    const int c = threadIdx.x;
-    const int r0 = blockIdx.x * 32;
-    float s = 0.f;
-    for (int r = r0; r < r0 + 32 && r < rows; r++) {
-        const size_t i = (size_t)r * kC + c;
-        const float v = dh[i] * dsilu_f(y[i]);
-        dy[i] = __float2bfloat16_rn(v);
-        s += v;
-    }
-    atomicAdd(&db[c], s);
-}
-
-// 32 x 32 tiled transpose: dst (cols x rows) = src (rows x cols)^T
-__global__ void k_transpose(const bf16 *__restrict__ src, int rows, int cols, bf16 *__restrict__ dst)
-{
-    __shared__ bf16 tile[32][33];
-    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;   // bx: column block, by: row block
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int r = by + j, c = bx + threadIdx.x;
-        if (r < rows && c < cols) tile[j][threadIdx.x] = src[(size_t)r * cols + c];
+    __shared__ bf16 tile[64][66];
+    const int bx = blockIdx.x * 64, by = blockIdx.y * 64;   // bx: column block, by: row block
+    const int part = threadIdx.x & 7, line = threadIdx.x >> 3;
+    for (int j = line; j < 64; j += 32) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(src + (size_t)(by + j) * cols + bx + 8 * part);
+        const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; k++) *reinterpret_cast<unsigned *>(&tile[j][8 * part + 2 * k]) = u[k];
     }
     __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += 8) {
-        const int c = bx + j, r = by + threadIdx.x;
-        if (r < rows && c < cols) dst[(size_t)c * rows + r] = tile[threadIdx.x][j];
+    for (int j = line; j < 64; j += 32) {
+        __align__(16) bf16 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) v[k] = tile[8 * part + k][j];
+        *reinterpret_cast<uint4 *>(dst + (size_t)(bx + j) * rows + by + 8 * part) = *reinterpret_cast<uint4 *>(v);
     }
 }
 
@@ -178,29 +276,53 @@ __global__ void k_transpose(const bf16 *__restrict__ src, int rows, int cols, bf
 // 2 dim columns and the loss sum; without t, out holds dout itself.
 // Writes dout in bf16 (rows x 64, zero elsewhere), its transpose (first
 // kNout rows of a 128 x np matrix) and the bias gradient.
+// (a row is 64 bytes: four loads; the bias gradient and the loss leave a warp as
+// one atomic each, not one per row: 117 -> 6.6 us on 19 072 rows)
 __global__ void k_output_grad(const float *__restrict__ out, const float *__restrict__ t,
                               const uint8_t *__restrict__ mask, int rows, int np, int nout, float inv_cnt,
                               bf16 *__restrict__ dout, bf16 *__restrict__ doutT, float *__restrict__ db,
                               float *__restrict__ loss)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    float L = 0.f;
+    float L = 0.f, d[kNout];
+#pragma unroll
+    for (int j = 0; j < kNout; j++) d[j] = 0.f;
     if (r < rows) {
         const float mk = t ? (mask ? (float)mask[r] : 1.0f) : 1.0f;
-        for (int j = 0; j < nout; j++) {
-            float d;
-            if (t) {
-                const float e = (out[(size_t)r * kNout + j] - t[(size_t)r * kNout + j]) * mk;
-                L += e * e;
-                d = 2.0f * e * inv_cnt;
-            } else {
-                d = out[(size_t)r * kNout + j];
-            }
-            const bf16 q = __float2bfloat16_rn(d);
-            dout[(size_t)r * kFin + j] = q;
-            doutT[(size_t)j * np + r] = q;
-            atomicAdd(&db[j], d);
+        float o[kNout], tt[kNout];
+#pragma unroll
+        for (int k = 0; k < kNout / 4; k++) {
+            const float4 v = reinterpret_cast<const float4 *>(out + (size_t)r * kNout)[k];
+            o[4 * k] = v.x, o[4 * k + 1] = v.y, o[4 * k + 2] = v.z, o[4 * k + 3] = v.w;
+            const float4 q = t ? reinterpret_cast<const float4 *>(t + (size_t)r * kNout)[k]
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+            tt[4 * k] = q.x, tt[4 * k + 1] = q.y, tt[4 * k + 2] = q.z, tt[4 * k + 3] = q.w;
         }
+        __align__(16) bf16 b[kNout];
+#pragma unroll
+        for (int j = 0; j < kNout; j++) {
+            if (j < nout) {
+                if (t) {
+                    const float e = (o[j] - tt[j]) * mk;
+                    L += e * e;
+                    d[j] = 2.0f * e * inv_cnt;
+                } else {
+                    d[j] = o[j];
+                }
+            }
+            b[j] = __float2bfloat16_rn(d[j]);
+            doutT[(size_t)j * np + r] = b[j];
+        }
+        uint4 *row = reinterpret_cast<uint4 *>(dout + (size_t)r * kFin);
+        row[0] = reinterpret_cast<uint4 *>(b)[0];
+        row[1] = reinterpret_cast<uint4 *>(b)[1];
+    }
+#pragma unroll
+    for (int j = 0; j < kNout; j++) {
+        if (j >= nout) break;
+        float v = d[j];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&db[j], v);
     }
     if (loss) {
         for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
@@ -223,17 +345,24 @@ __global__ void k_adam(float *__restrict__ th, const float *__restrict__ gr, flo
     th[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
 }
 
-// bf16 weight copies: W (out x in) as is, and W^T (in x out) padded to ldT
-// columns (zeros beyond out)
-__global__ void k_weights(const float *__restrict__ W, int out, int in, bf16 *__restrict__ Wb, bf16 *__restrict__ WT,
-                          int ldT)
+// bf16 weight copies of all layers in one launch: W (out x in) as is, and W^T
+// (in x out) padded to ldT columns (zeros beyond out); blockIdx.y picks the layer
+struct WeightCopy {
+    const float *W;
+    bf16 *Wb, *WT;
+    int out, in, ldT;
+};
+struct WeightCopies {
+    WeightCopy l[kLayers + 2];
+};
+__global__ void k_weights(const __grid_constant__ WeightCopies all)
 {
+    const WeightCopy &l = all.l[blockIdx.y];
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= out * in) return;
-    const int o = t / in, i = t % in;
-    const bf16 q = __float2bfloat16_rn(W[t]);
-    if (Wb) Wb[t] = q;
-    if (WT) WT[(size_t)i * ldT + o] = q;
+    if (t >= l.out * l.in) return;
+    const bf16 q = __float2bfloat16_rn(l.W[t]);
+    l.Wb[t] = q;
+    if (l.WT) l.WT[(size_t)(t % l.in) * l.ldT + t / l.in] = q;
 }
 
 inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
@@ -299,11 +428,11 @@ int refresh_weights(sphfsi_mpnn *m)
 {
     const Layout &L = m->L;
     cudaStream_t st = m->st;
-    k_weights<<<nblk(kC * kFin, 256), 256, 0, st>>>(m->theta + L.enc_W, kC, kFin, m->Wenc, nullptr, 0);
-    for (int l = 0; l < kLayers; l++)
-        k_weights<<<nblk((long long)kC * m->zd, 256), 256, 0, st>>>(m->theta + L.W[l], kC, m->zd, m->Wl[l], m->WlT[l],
-                                                                     kC);
-    k_weights<<<nblk(kNout * kC, 256), 256, 0, st>>>(m->theta + L.dec_W, kNout, kC, m->Wdec, m->WdecT, kFin);
+    WeightCopies all;
+    all.l[0] = {m->theta + L.enc_W, m->Wenc, nullptr, kC, kFin, 0};
+    for (int l = 0; l < kLayers; l++) all.l[1 + l] = {m->theta + L.W[l], m->Wl[l], m->WlT[l], kC, m->zd, kC};
+    all.l[kLayers + 1] = {m->theta + L.dec_W, m->Wdec, m->WdecT, kNout, kC, kFin};
+    k_weights<<<dim3(nblk((long long)kC * m->zd, 256), kLayers + 2), 256, 0, st>>>(all);
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;
 }
 
@@ -312,18 +441,20 @@ int forward(sphfsi_mpnn *m)
     cudaStream_t st = m->st;
     const Layout &L = m->L;
     const long long np = m->np, nn = m->nn;
-    k_to_bf16<<<nblk(nn * kFin, 256), 256, 0, st>>>(m->xin, kFin, (int)nn, kFin, m->xb, kFin);
+    k_to_bf16<<<nblk(nn * kFin / 4, 256), 256, 0, st>>>((const float4 *)m->xin, nn * kFin / 4, (uint2 *)m->xb);
     LTRY(gemm(m, m->xb, m->Wenc, m->theta + L.enc_b, m->yenc, np, kC, kFin));
-    k_act<<<nblk(np * kC, 256), 256, 0, st>>>(m->yenc, m->h, np * kC, 0);
+    k_act<<<nblk(np * kC / 4, 256), 256, 0, st>>>((const float4 *)m->yenc, (float4 *)m->h, np * kC / 4, 0);
     for (int l = 0; l < kLayers; l++) {
         if (m->dim == 2)
-            k_aggregate<2><<<(int)nn, kC, 0, st>>>(m->h, m->zb[l], m->n, m->ptr, m->idx, m->w, m->g);
+            k_aggregate<2><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
+                                                                     m->ptr, m->idx, m->w, m->g);
         else
-            k_aggregate<3><<<(int)nn, kC, 0, st>>>(m->h, m->zb[l], m->n, m->ptr, m->idx, m->w, m->g);
+            k_aggregate<3><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
+                                                                     m->ptr, m->idx, m->w, m->g);
         LTRY(gemm(m, m->zb[l], m->Wl[l], m->theta + L.b[l], m->y[l], np, kC, m->zd));
-        k_act<<<nblk(np * kC, 256), 256, 0, st>>>(m->y[l], m->h, np * kC, 1);
+        k_act<<<nblk(np * kC / 4, 256), 256, 0, st>>>((const float4 *)m->y[l], (float4 *)m->h, np * kC / 4, 1);
     }
-    k_to_bf16<<<nblk(nn * kC, 256), 256, 0, st>>>(m->h, kC, (int)nn, kC, m->hb, kC);
+    k_to_bf16<<<nblk(nn * kC / 4, 256), 256, 0, st>>>((const float4 *)m->h, nn * kC / 4, (uint2 *)m->hb);
     LTRY(gemm(m, m->hb, m->Wdec, m->theta + L.dec_b, m->out, np, kNout, kC));
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;
 }
@@ -335,14 +466,13 @@ int backward(sphfsi_mpnn *m, const float *dout_or_out, const float *t, const uin
     cudaStream_t st = m->st;
     const Layout &L = m->L;
     const long long np = m->np, nn = m->nn;
-    const dim3 tb(32, 8);
     LTRY(cudaMemsetAsync(m->grad, 0, sizeof(float) * L.total, st) == cudaSuccess ? 0 : SPHFSI_E_CUDA);
     if (loss) LTRY(cudaMemsetAsync(loss, 0, sizeof(float), st) == cudaSuccess ? 0 : SPHFSI_E_CUDA);
     k_output_grad<<<nblk(nn, 128), 128, 0, st>>>(dout_or_out, t, mask, (int)nn, (int)np, t ? 2 * m->dim : kNout,
                                                  inv_cnt,
                                                  m->doutb, m->doutT, m->grad + L.dec_b, loss);
     // decoder: dW_dec = dout^T h (first kNout rows of a 128-row product), dh = dout W_dec
-    k_transpose<<<dim3(kC / 32, (unsigned)(np / 32)), tb, 0, st>>>(m->hb, (int)np, kC, m->hT);
+    k_transpose<<<dim3(kC / 64, (unsigned)(np / 64)), 256, 0, st>>>(m->hb, (int)np, kC, m->hT);
     LTRY(gemm(m, m->doutT, m->hT, nullptr, m->dwdec, kC, kC, np));
     LTRY(cudaMemcpyAsync(m->grad + L.dec_W, m->dwdec, sizeof(float) * kNout * kC, cudaMemcpyDeviceToDevice, st) ==
                  cudaSuccess
@@ -350,20 +480,22 @@ int backward(sphfsi_mpnn *m, const float *dout_or_out, const float *t, const uin
              : SPHFSI_E_CUDA);
     LTRY(gemm(m, m->doutb, m->WdecT, nullptr, m->dh, np, kC, kFin));
     for (int l = kLayers - 1; l >= 0; l--) {
-        k_dsilu<<<(unsigned)(np / 32), kC, 0, st>>>(m->dh, m->y[l], (int)nn, m->dyb, m->grad + L.b[l]);
-        k_transpose<<<dim3(kC / 32, (unsigned)(np / 32)), tb, 0, st>>>(m->dyb, (int)np, kC, m->dyT);
-        k_transpose<<<dim3((unsigned)(m->zd / 32), (unsigned)(np / 32)), tb, 0, st>>>(m->zb[l], (int)np, m->zd,
+        k_dsilu<<<(unsigned)std::min(np / 32, 304LL), 256, 0, st>>>((const float4 *)m->dh, (const float4 *)m->y[l], (int)nn, (int)np,
+                                                     (uint2 *)m->dyb, m->dyT, m->grad + L.b[l]);
+        k_transpose<<<dim3((unsigned)(m->zd / 64), (unsigned)(np / 64)), 256, 0, st>>>(m->zb[l], (int)np, m->zd,
                                                                                         m->zT);
         LTRY(gemm(m, m->dyT, m->zT, nullptr, m->grad + L.W[l], kC, m->zd, np));
         LTRY(gemm(m, m->dyb, m->WlT[l], nullptr, m->dz, np, m->zd, kC));
         if (m->dim == 2)
-            k_agg_adjoint<2><<<(int)nn, kC, 0, st>>>(m->dz, m->dh, m->n, m->ptr, m->idx, m->w, m->g);
+            k_agg_adjoint<2><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
+                                                                       m->ptr, m->idx, m->w, m->g);
         else
-            k_agg_adjoint<3><<<(int)nn, kC, 0, st>>>(m->dz, m->dh, m->n, m->ptr, m->idx, m->w, m->g);
+            k_agg_adjoint<3><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
+                                                                       m->ptr, m->idx, m->w, m->g);
     }
-    k_dsilu<<<(unsigned)(np / 32), kC, 0, st>>>(m->dh, m->yenc, (int)nn, m->dyb, m->grad + L.enc_b);
-    k_transpose<<<dim3(kC / 32, (unsigned)(np / 32)), tb, 0, st>>>(m->dyb, (int)np, kC, m->dyT);
-    k_transpose<<<dim3(kFin / 32, (unsigned)(np / 32)), tb, 0, st>>>(m->xb, (int)np, kFin, m->xT);
+    k_dsilu<<<(unsigned)std::min(np / 32, 304LL), 256, 0, st>>>((const float4 *)m->dh, (const float4 *)m->yenc, (int)nn, (int)np,
+                                                 (uint2 *)m->dyb, m->dyT, m->grad + L.enc_b);
+    k_transpose<<<dim3(kFin / 64, (unsigned)(np / 64)), 256, 0, st>>>(m->xb, (int)np, kFin, m->xT);
     LTRY(gemm(m, m->dyT, m->xT, nullptr, m->grad + L.enc_W, kC, kFin, np));
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;
 }
