@@ -43,11 +43,11 @@ __device__ __forceinline__ void pdl_enter()
 }
 
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_k(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem,
+static inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem,
                                    cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;

@@ -76,6 +76,7 @@ __device__ __forceinline__ uint2 pack4(float4 v)
 // dst = bf16(src), 4 n4 values
 __global__ void k_to_bf16(const float4 *__restrict__ src, long long n4, uint2 *__restrict__ dst)
 {
+    pdl_enter();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n4) dst[t] = pack4(src[t]);
 }
@@ -83,6 +84,7 @@ __global__ void k_to_bf16(const float4 *__restrict__ src, long long n4, uint2 *_
 // mode 0: h = silu(y); mode 1: h += silu(y) (4 n4 values)
 __global__ void k_act(const float4 *__restrict__ y, float4 *__restrict__ h, long long n4, int mode)
 {
+    pdl_enter();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n4) return;
     const float4 v = y[t];
@@ -127,6 +129,7 @@ __global__ void __launch_bounds__(32 * kNodes) k_aggregate(const float4 *__restr
                                                            const int *__restrict__ idx, const float *__restrict__ w,
                                                            const float *__restrict__ g)
 {
+    pdl_enter();
     constexpr int C4 = kC / 4;
     const int a = blockIdx.x * kNodes + (int)(threadIdx.x >> 5), c = threadIdx.x & 31;
     if (a >= nn) return;
@@ -168,6 +171,7 @@ __global__ void __launch_bounds__(32 * kNodes) k_agg_adjoint(const float4 *__res
                                                              const int *__restrict__ idx, const float *__restrict__ w,
                                                              const float *__restrict__ g)
 {
+    pdl_enter();
     constexpr int C4 = kC / 4, Z4 = C4 * (2 + D), U = 2;
     const int b = blockIdx.x * kNodes + (int)(threadIdx.x >> 5), c = threadIdx.x & 31;
     if (b >= nn) return;
@@ -214,6 +218,7 @@ __global__ void __launch_bounds__(256) k_dsilu(const float4 *__restrict__ dh, co
                                                int np, uint2 *__restrict__ dy, bf16 *__restrict__ dyT,
                                                float *__restrict__ db)
 {
+    pdl_enter();
     constexpr int C4 = kC / 4;
     __shared__ __align__(16) float s_sum[8][kC];
     __shared__ __align__(8) bf16 s_dy[32][kC + 4];
@@ -254,6 +259,7 @@ __global__ void __launch_bounds__(256) k_dsilu(const float4 *__restrict__ dh, co
 __global__ void __launch_bounds__(256) k_transpose(const bf16 *__restrict__ src, int rows, int cols,
                                                    bf16 *__restrict__ dst)
 {
+    pdl_enter();
     __shared__ bf16 tile[64][66];
     const int bx = blockIdx.x * 64, by = blockIdx.y * 64;   // bx: column block, by: row block
     const int part = threadIdx.x & 7, line = threadIdx.x >> 3;
@@ -283,6 +289,7 @@ __global__ void k_output_grad(const float *__restrict__ out, const float *__rest
                               bf16 *__restrict__ dout, bf16 *__restrict__ doutT, float *__restrict__ db,
                               float *__restrict__ loss)
 {
+    pdl_enter();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     float L = 0.f, d[kNout];
 #pragma unroll
@@ -335,6 +342,7 @@ __global__ void k_output_grad(const float *__restrict__ out, const float *__rest
 __global__ void k_adam(float *__restrict__ th, const float *__restrict__ gr, float *__restrict__ m,
                        float *__restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1, float c2)
 {
+    pdl_enter();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float g = gr[i];
@@ -357,6 +365,7 @@ struct WeightCopies {
 };
 __global__ void k_weights(const __grid_constant__ WeightCopies all)
 {
+    pdl_enter();
     const WeightCopy &l = all.l[blockIdx.y];
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= l.out * l.in) return;
@@ -432,7 +441,7 @@ int refresh_weights(sphfsi_mpnn *m)
     all.l[0] = {m->theta + L.enc_W, m->Wenc, nullptr, kC, kFin, 0};
     for (int l = 0; l < kLayers; l++) all.l[1 + l] = {m->theta + L.W[l], m->Wl[l], m->WlT[l], kC, m->zd, kC};
     all.l[kLayers + 1] = {m->theta + L.dec_W, m->Wdec, m->WdecT, kNout, kC, kFin};
-    k_weights<<<dim3(nblk((long long)kC * m->zd, 256), kLayers + 2), 256, 0, st>>>(all);
+    launch_k(k_weights, dim3(nblk((long long)kC * m->zd, 256), kLayers + 2), 256, 0, st, all);
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;
 }
 
@@ -441,20 +450,20 @@ int forward(sphfsi_mpnn *m)
     cudaStream_t st = m->st;
     const Layout &L = m->L;
     const long long np = m->np, nn = m->nn;
-    k_to_bf16<<<nblk(nn * kFin / 4, 256), 256, 0, st>>>((const float4 *)m->xin, nn * kFin / 4, (uint2 *)m->xb);
+    launch_k(k_to_bf16, nblk(nn * kFin / 4, 256), 256, 0, st, (const float4 *)m->xin, nn * kFin / 4, (uint2 *)m->xb);
     LTRY(gemm(m, m->xb, m->Wenc, m->theta + L.enc_b, m->yenc, np, kC, kFin));
-    k_act<<<nblk(np * kC / 4, 256), 256, 0, st>>>((const float4 *)m->yenc, (float4 *)m->h, np * kC / 4, 0);
+    launch_k(k_act, nblk(np * kC / 4, 256), 256, 0, st, (const float4 *)m->yenc, (float4 *)m->h, np * kC / 4, 0);
     for (int l = 0; l < kLayers; l++) {
         if (m->dim == 2)
-            k_aggregate<2><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
+            launch_k(k_aggregate<2>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
                                                                      m->ptr, m->idx, m->w, m->g);
         else
-            k_aggregate<3><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
+            launch_k(k_aggregate<3>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
                                                                      m->ptr, m->idx, m->w, m->g);
         LTRY(gemm(m, m->zb[l], m->Wl[l], m->theta + L.b[l], m->y[l], np, kC, m->zd));
-        k_act<<<nblk(np * kC / 4, 256), 256, 0, st>>>((const float4 *)m->y[l], (float4 *)m->h, np * kC / 4, 1);
+        launch_k(k_act, nblk(np * kC / 4, 256), 256, 0, st, (const float4 *)m->y[l], (float4 *)m->h, np * kC / 4, 1);
     }
-    k_to_bf16<<<nblk(nn * kC / 4, 256), 256, 0, st>>>((const float4 *)m->h, nn * kC / 4, (uint2 *)m->hb);
+    launch_k(k_to_bf16, nblk(nn * kC / 4, 256), 256, 0, st, (const float4 *)m->h, nn * kC / 4, (uint2 *)m->hb);
     LTRY(gemm(m, m->hb, m->Wdec, m->theta + L.dec_b, m->out, np, kNout, kC));
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;
 }
@@ -468,11 +477,11 @@ int backward(sphfsi_mpnn *m, const float *dout_or_out, const float *t, const uin
     const long long np = m->np, nn = m->nn;
     LTRY(cudaMemsetAsync(m->grad, 0, sizeof(float) * L.total, st) == cudaSuccess ? 0 : SPHFSI_E_CUDA);
     if (loss) LTRY(cudaMemsetAsync(loss, 0, sizeof(float), st) == cudaSuccess ? 0 : SPHFSI_E_CUDA);
-    k_output_grad<<<nblk(nn, 128), 128, 0, st>>>(dout_or_out, t, mask, (int)nn, (int)np, t ? 2 * m->dim : kNout,
+    launch_k(k_output_grad, nblk(nn, 128), 128, 0, st, dout_or_out, t, mask, (int)nn, (int)np, t ? 2 * m->dim : kNout,
                                                  inv_cnt,
                                                  m->doutb, m->doutT, m->grad + L.dec_b, loss);
     // decoder: dW_dec = dout^T h (first kNout rows of a 128-row product), dh = dout W_dec
-    k_transpose<<<dim3(kC / 64, (unsigned)(np / 64)), 256, 0, st>>>(m->hb, (int)np, kC, m->hT);
+    launch_k(k_transpose, dim3(kC / 64, (unsigned)(np / 64)), 256, 0, st, m->hb, (int)np, kC, m->hT);
     LTRY(gemm(m, m->doutT, m->hT, nullptr, m->dwdec, kC, kC, np));
     LTRY(cudaMemcpyAsync(m->grad + L.dec_W, m->dwdec, sizeof(float) * kNout * kC, cudaMemcpyDeviceToDevice, st) ==
                  cudaSuccess
@@ -480,22 +489,22 @@ int backward(sphfsi_mpnn *m, const float *dout_or_out, const float *t, const uin
              : SPHFSI_E_CUDA);
     LTRY(gemm(m, m->doutb, m->WdecT, nullptr, m->dh, np, kC, kFin));
     for (int l = kLayers - 1; l >= 0; l--) {
-        k_dsilu<<<(unsigned)std::min(np / 32, 304LL), 256, 0, st>>>((const float4 *)m->dh, (const float4 *)m->y[l], (int)nn, (int)np,
+        launch_k(k_dsilu, (unsigned)std::min(np / 32, 304LL), 256, 0, st, (const float4 *)m->dh, (const float4 *)m->y[l], (int)nn, (int)np,
                                                      (uint2 *)m->dyb, m->dyT, m->grad + L.b[l]);
-        k_transpose<<<dim3((unsigned)(m->zd / 64), (unsigned)(np / 64)), 256, 0, st>>>(m->zb[l], (int)np, m->zd,
+        launch_k(k_transpose, dim3((unsigned)(m->zd / 64), (unsigned)(np / 64)), 256, 0, st, m->zb[l], (int)np, m->zd,
                                                                                         m->zT);
         LTRY(gemm(m, m->dyT, m->zT, nullptr, m->grad + L.W[l], kC, m->zd, np));
         LTRY(gemm(m, m->dyb, m->WlT[l], nullptr, m->dz, np, m->zd, kC));
         if (m->dim == 2)
-            k_agg_adjoint<2><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
+            launch_k(k_agg_adjoint<2>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
                                                                        m->ptr, m->idx, m->w, m->g);
         else
-            k_agg_adjoint<3><<<nblk(nn, kNodes), 32 * kNodes, 0, st>>>((const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
+            launch_k(k_agg_adjoint<3>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
                                                                        m->ptr, m->idx, m->w, m->g);
     }
-    k_dsilu<<<(unsigned)std::min(np / 32, 304LL), 256, 0, st>>>((const float4 *)m->dh, (const float4 *)m->yenc, (int)nn, (int)np,
+    launch_k(k_dsilu, (unsigned)std::min(np / 32, 304LL), 256, 0, st, (const float4 *)m->dh, (const float4 *)m->yenc, (int)nn, (int)np,
                                                  (uint2 *)m->dyb, m->dyT, m->grad + L.enc_b);
-    k_transpose<<<dim3(kFin / 64, (unsigned)(np / 64)), 256, 0, st>>>(m->xb, (int)np, kFin, m->xT);
+    launch_k(k_transpose, dim3(kFin / 64, (unsigned)(np / 64)), 256, 0, st, m->xb, (int)np, kFin, m->xT);
     LTRY(gemm(m, m->dyT, m->xT, nullptr, m->grad + L.enc_W, kC, kFin, np));
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;
 }
@@ -696,7 +705,7 @@ int sphfsi_mpnn_train_step(sphfsi_mpnn *m, const float *x, const float *target, 
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = (float)(1.0 / (1.0 - std::pow(0.9, (double)m->step)));
     const float c2 = (float)(1.0 / (1.0 - std::pow(0.999, (double)m->step)));
-    k_adam<<<nblk(m->L.total, 256), 256, 0, m->st>>>(m->theta, m->grad, m->am, m->av, m->L.total, lr, b1, b2, 1e-8f,
+    launch_k(k_adam, nblk(m->L.total, 256), 256, 0, m->st, m->theta, m->grad, m->am, m->av, m->L.total, lr, b1, b2, 1e-8f,
                                                      c1, c2);
     LTRY(refresh_weights(m));
     if (loss && cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDefault, m->st) != cudaSuccess)

@@ -23,7 +23,8 @@
 // of operand reads against 512 cycles of MMA, which bounds large products:
 // 4096 x 4096 x 4096 takes 124 us (1.11 PFLOP/s; 312 us with the idle lanes of
 // warps 0 and 1 spinning next to their lane 0 and a row of 16-byte stores per
-// lane), 16384 x 256 x 4096 48 us (85).  Sharing B in clusters of 2 or 4 by
+// lane), 16384 x 256 x 4096 46 us (85), and less with a pair of CTAs (below).
+// Sharing B in clusters of 2 or 4 by
 // multicast, prefetching A into L2 and 256-byte L2 promotion change neither.
 // Every wait is bounded; a timeout sets a status bit, skips the epilogue and
 // still frees the tensor memory.
@@ -89,12 +90,61 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr)
 constexpr int kStages = 4;
 constexpr int kEpiLd = 36;   // floats per row of a warp's 32 x 32 epilogue block (16-byte rows, 8 lanes without conflicts)
 
+// the 128 x NT accumulator at tmem (+ bias) to rows m0.., columns n0.. of C
+template <int NT>
+__device__ __forceinline__ void store_tile(uint32_t tmem, float *ring, const float *__restrict__ bias,
+                                           float *__restrict__ C, int N, int m0, int n0)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int CW = NT < 32 ? NT : 32;   // columns per block
+    constexpr int kLn = CW / 4, kRw = 32 / kLn;   // lanes per row, rows per store
+    float *blk = ring + warp * (32 * kEpiLd);
+    const int cc = 4 * (lane % kLn), rr = lane / kLn;
+#pragma unroll 1
+    for (int c = 0; c < NT; c += CW) {
+#pragma unroll
+        for (int h = 0; h < CW; h += 16) {
+            uint32_t v[16];
+            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c + h);
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                "%13, %14, %15}, [%16];"
+                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+                  "=r"(v[15])
+                : "r"(taddr));
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                *reinterpret_cast<uint4 *>(blk + lane * kEpiLd + h + 4 * j) =
+                    make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+        __syncwarp();
+        float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (bias) bv = make_float4(bias[n0 + c + cc], bias[n0 + c + cc + 1], bias[n0 + c + cc + 2],
+                                   bias[n0 + c + cc + 3]);
+#pragma unroll
+        for (int k = 0; k < 32; k += kRw) {
+            float4 o = *reinterpret_cast<const float4 *>(blk + (k + rr) * kEpiLd + cc);
+            if (bias) {
+                o.x += bv.x;
+                o.y += bv.y;
+                o.z += bv.z;
+                o.w += bv.w;
+            }
+            *reinterpret_cast<float4 *>(C + (size_t)(m0 + warp * 32 + k + rr) * N + n0 + c + cc) = o;
+        }
+        __syncwarp();
+    }
+}
+
 template <int NT>
 __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant__ CUtensorMap tmA,
                                                           const __grid_constant__ CUtensorMap tmB,
                                                           const float *__restrict__ bias, float *__restrict__ C,
                                                           int M, int N, int K, int kper, int stages)
 {
+    pdl_enter();
     // split K: slice blockIdx.z covers chunks [z kper, (z + 1) kper) and
     // writes its partial tile to C + z M N (the caller reduces the slices)
     C += (size_t)blockIdx.z * M * N;
@@ -191,52 +241,146 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_bf16(const __grid_constant_
     if (!ok && tid == 0) atomicOr(&g_tc_status, 1u);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
-        constexpr int CW = NT < 32 ? NT : 32;   // columns per block
-        constexpr int kLn = CW / 4, kRw = 32 / kLn;   // lanes per row, rows per store
-        float *blk = reinterpret_cast<float *>(dsm + (base - smem_u32(dsm))) + warp * (32 * kEpiLd);
-        const int cc = 4 * (lane % kLn), rr = lane / kLn;
-#pragma unroll 1
-        for (int c = 0; c < NT; c += CW) {
-#pragma unroll
-            for (int h = 0; h < CW; h += 16) {
-                uint32_t v[16];
-                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c + h);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-                    "%13, %14, %15}, [%16];"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                      "=r"(v[15])
-                    : "r"(taddr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                for (int j = 0; j < 4; j++)
-                    *reinterpret_cast<uint4 *>(blk + lane * kEpiLd + h + 4 * j) =
-                        make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            }
-            __syncwarp();
-            float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (bias) bv = make_float4(bias[n0 + c + cc], bias[n0 + c + cc + 1], bias[n0 + c + cc + 2],
-                                       bias[n0 + c + cc + 3]);
-#pragma unroll
-            for (int k = 0; k < 32; k += kRw) {
-                float4 o = *reinterpret_cast<const float4 *>(blk + (k + rr) * kEpiLd + cc);
-                if (bias) {
-                    o.x += bv.x;
-                    o.y += bv.y;
-                    o.z += bv.z;
-                    o.w += bv.w;
-                }
-                *reinterpret_cast<float4 *>(C + (size_t)(m0 + warp * 32 + k + rr) * N + n0 + c + cc) = o;
-            }
-            __syncwarp();
-        }
+        store_tile<NT>(tmem, reinterpret_cast<float *>(dsm + (base - smem_u32(dsm))), bias, C, N, m0, n0);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 2) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+    }
+}
+
+// The same product with a pair of CTAs (a cluster of 2, cta_group::2) on a
+// 256 x 256 tile: each loads its 128 rows of A and half of B (128 rows), the
+// first one's MMAs read both halves (M = 256) and leave 128 rows in either
+// CTA's tensor memory.  B is then written to and read from each shared memory
+// once per two tiles: 4096 x 4096 x 4096 124 -> 117 us (1.17 PFLOP/s).  One pair
+// fills its SMs' shared memory, so pairs never wait for each other's tensor memory.
+//
+// Both CTAs' loads complete on the first one's "full" mbarrier, which it arms
+// with the bytes of both; a commit frees the stage in both.
+constexpr int kPairStages = 6;
+constexpr int kPairStage = 2 * kAStage;   // 128 x 64 of A and of B
+
+__device__ __forceinline__ uint32_t cta0_addr(uint32_t a)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
+    return r;
+}
+__device__ __forceinline__ void pair_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void pair_load(uint32_t dst, const CUtensorMap *tm, int x, int y, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+        "%3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void pair_commit(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::
+                     "r"(bar),
+                 "h"((uint16_t)3)
+                 : "memory");
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads)
+    k_gemm_bf16_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                     const float *__restrict__ bias, float *__restrict__ C, int N, int nk)
+{
+    pdl_enter();
+    extern __shared__ uint8_t dsm[];
+    __shared__ __align__(8) uint64_t full[kPairStages], empty[kPairStages], done;
+    __shared__ uint32_t s_tmem;
+    const uint32_t base = (smem_u32(dsm) + 1023u) & ~1023u;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x & 1, m0 = blockIdx.x * 128, n0 = blockIdx.y * 256;
+
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&s_tmem))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < kPairStages; s++) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[s])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[s])) : "memory");
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&done)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    pair_sync();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem;
+
+    bool ok = true;
+    if (warp == 0 && lane == 0) {
+        uint32_t ph = 1u;
+        int s = 0;
+        for (int kc = 0; kc < nk; kc++) {
+            if (!mbar_wait(smem_u32(&empty[s]), ph)) {
+                ok = false;
+                break;
+            }
+            const uint32_t a_s = base + s * kPairStage, fb = cta0_addr(smem_u32(&full[s]));
+            if (rank == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&full[s])),
+                             "r"(2 * kPairStage)
+                             : "memory");
+            pair_load(a_s, &tmA, kc * kKChunk, m0, fb);
+            pair_load(a_s + kAStage, &tmB, kc * kKChunk, n0 + rank * 128, fb);
+            if (++s == kPairStages) s = 0, ph ^= 1u;
+        }
+        // every commit has arrived here before this CTA may leave
+        for (int k = 0; ok && k < min(nk, kPairStages); k++) {
+            if (s == 0) s = kPairStages, ph ^= 1u;
+            s--;
+            ok = mbar_wait(smem_u32(&empty[s]), ph ^ 1u);
+        }
+    } else if (rank == 0 && warp == 1 && lane == 0) {
+        uint32_t ph = 0u;
+        for (int kc = 0, s = 0; kc < nk; kc++) {
+            if (!mbar_wait(smem_u32(&full[s]), ph)) {
+                ok = false;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = base + s * kPairStage, b0 = a0 + kAStage;
+#pragma unroll
+            for (int kk = 0; kk < kKChunk / 16; kk++) {
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\t"
+                    "setp.ne.b32 p, %4, 0;\n\t"
+                    "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+                    "l"(sdesc_sw128(a0 + kk * 32)), "l"(sdesc_sw128(b0 + kk * 32)), "r"(idesc_bf16(256, 256)),
+                    "r"((kc | kk) ? 1u : 0u)
+                    : "memory");
+            }
+            pair_commit(smem_u32(&empty[s]));
+            if (++s == kPairStages) s = 0, ph ^= 1u;
+        }
+        pair_commit(smem_u32(&done));
+    }
+    __syncwarp();
+    if (!mbar_wait(smem_u32(&done), 0u)) ok = false;
+    ok = __syncthreads_and(ok);
+    if (!ok && tid == 0) atomicOr(&g_tc_status, 1u);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok) store_tile<256>(tmem, reinterpret_cast<float *>(dsm + (base - smem_u32(dsm))), bias, C, N, m0, n0);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    pair_sync();
+    if (warp == 2) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
     }
 }
 
@@ -281,6 +425,7 @@ int make_map(CUtensorMap *m, const void *ptr, long long rows, long long cols, in
 __global__ void k_splitk_sum(const float *__restrict__ ws, int S, long long MN, int N, const float *__restrict__ bias,
                              float *__restrict__ C)
 {
+    pdl_enter();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MN) return;
     float v = bias ? bias[i % N] : 0.0f;
@@ -331,12 +476,30 @@ int launch_tile(const uint16_t *A, const uint16_t *B, const float *bias, float *
     // the SM (19072 x 512 x 128: 12.3 -> 11.0 us)
     const int stages = std::min(kStages, kper), smem = stages * kStage + 1024;
     const dim3 grid(M / 128, N / NT, S);
-    k_gemm_bf16<NT><<<grid, kTcThreads, smem, st>>>(ta, tb, S == 1 ? bias : nullptr, S == 1 ? C : g_ws, M, N, K, kper,
+    launch_k(k_gemm_bf16<NT>, grid, kTcThreads, smem, st, ta, tb, S == 1 ? bias : nullptr, S == 1 ? C : g_ws, M, N, K, kper,
                                                     stages);
     if (S > 1) {
         const long long MN = (long long)M * N;
-        k_splitk_sum<<<(unsigned)((MN + 255) / 256), 256, 0, st>>>(g_ws, S, MN, N, bias, C);
+        launch_k(k_splitk_sum, (unsigned)((MN + 255) / 256), 256, 0, st, g_ws, S, MN, N, bias, C);
     }
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+int launch_pair(const uint16_t *A, const uint16_t *B, const float *bias, float *C, int M, int N, int K,
+                cudaStream_t st)
+{
+    const int smem = kPairStages * kPairStage + 1024;
+    static bool attr_set = false;
+    if (!attr_set) {
+        if (cudaFuncSetAttribute(k_gemm_bf16_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+            return -3;
+        attr_set = true;
+    }
+    alignas(64) CUtensorMap ta, tb;
+    int rc = make_map(&ta, A, M, K, 128);
+    if (!rc) rc = make_map(&tb, B, N, K, 128);
+    if (rc) return rc;
+    launch_k(k_gemm_bf16_pair, dim3(M / 128, N / 256), kTcThreads, smem, st, ta, tb, bias, C, N, K / kKChunk);
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -349,6 +512,12 @@ int launch_gemm_bf16(const uint16_t *A, const uint16_t *B, const float *bias, fl
     if (M / 128 > 65535 * 1024LL || K > (1LL << 30) || N > (1LL << 30)) return -7;
     if (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & 15) return -1;
     const int m = (int)M, n = (int)N, k = (int)K;
+    // pairs of CTAs for a long K loop that needs no split: 16384 x 256 x 4096 45.8 ->
+    // 43.6 us, 9728 x 256 x 4096 39.6 -> 37.5, 2560 x 1024 x 2048 25.3 -> 23.2; with
+    // K = 1024 they lose (20480 x 512: 45.7 -> 49.8), as the one tile per SM then
+    // leaves its epilogue uncovered
+    if (n % 256 == 0 && m % 256 == 0 && k >= 32 * kKChunk && (long long)(m / 128) * (n / 256) >= 76)
+        return launch_pair(A, B, bias, C, m, n, k, st);
     if (n % 256 == 0) return launch_tile<256>(A, B, bias, C, m, n, k, st);
     if (n % 128 == 0) return launch_tile<128>(A, B, bias, C, m, n, k, st);
     if (n % 64 == 0) return launch_tile<64>(A, B, bias, C, m, n, k, st);
