@@ -156,7 +156,8 @@ KERNEL_SOURCE = {"k_momentum": "sph_fluid.cu", "k_solid_fluid_force": "sph_fluid
                  "k_solid_cluster2d_one": "sph_solid.cu", "k_solid_cluster2d": "sph_solid.cu",
                  "k_solid_cluster2d_1b": "sph_solid.cu",
                  "k_solid_cluster_one": "sph_solid.cu", "k_solid_cluster": "sph_solid.cu",
-                 "k_solid_substeps": "sph_solid.cu", "k_gemm_bf16": "sph_learn_gemm.cu",
+                 "k_solid_substeps": "sph_solid.cu", "k_solid_window": "sph_solid.cu",
+                 "k_gemm_bf16": "sph_learn_gemm.cu",
                  "k_pairlist": "sph_fluid.cu"}
 
 
@@ -418,7 +419,8 @@ def run_gpu(args, rank, world, local_rank):
         solid_kernel = "k_solid_cluster2d" if two_d else "k_solid_cluster"
     else:
         solid_kernel = {1: "k_solid_cluster2d_one" if two_d else "k_solid_cluster_one",
-                        2: "k_solid_substeps", 3: "k_solid_cluster2d_1b"}.get(info1["solid_path"], "k_solid_substeps")
+                        # (the windowed form; k_solid_substeps where its windows do not fit)
+                        2: "k_solid_window", 3: "k_solid_cluster2d_1b"}.get(info1["solid_path"], "k_solid_window")
     kernel_names = {"solid_substeps": solid_kernel, "momentum": "k_momentum", "continuity": "k_density",
                     "neighbour_rows": "k_pairlist",
                     "solid_fluid_force": "k_solid_fluid_force", "reinit": "k_reinit",

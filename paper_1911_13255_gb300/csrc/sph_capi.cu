@@ -1190,12 +1190,14 @@ int sphfsi_finalize(sphfsi_ctx *c)
     TRY(dalloc(c, &F.gbar, 2));
     // neighbour rows (tuned): about 20 (2-D) or 80 (3-D) neighbours per fluid
     // particle on a lattice, wall neighbours included.  On from 32 768 fluid
-    // particles in 2-D (2 lanes per target) and 16 384 in 3-D (4): below, the
-    // loops are too short to pay for the build.  Step with the cell form and
-    // with rows: 2-D channels of 10k, 40k and 79k particles 67, 80 and 146 us
-    // against 62, 76 and 108; batches of 28k, 171k and 577k 130, 248 and 574
-    // against 138, 234 and 485; 3-D tanks of 6k, 17k, 62k and 175k 230, 257, 393
-    // and 780 against 241, 246, 320 and 476.
+    // particles in 2-D (2 lanes per target) and 16 384 in 3-D (4).  Step with the
+    // cell form and with rows: 2-D channels of 33k particles 87 against 71 us,
+    // batches of 171k and 577k 248 and 574 against 234 and 485; 3-D tanks of 4k,
+    // 11k, 24k and 62k 219, 151, 202 and 393 against 218, 151, 182 and 320.
+    // Smaller 2-D contexts would gain too (a channel of 10k 65 -> 60 us, a dam
+    // break of 14k 90 -> 87), but the form decides the order of the sums, and a
+    // batch of a few thousand particles per instance equals its instances
+    // stepped alone to the last bit: both have to take the same one.
     F.n = (int)nf;
     c->S.n = (int)ns;
     cell_form(c, F);
