@@ -295,9 +295,11 @@ __device__ __forceinline__ void reinit_finish(const Batch &bt, const Fluid &f, i
 // a warp each, in the first blocks (as in k_momentum; the walls, whose pairs
 // cost no more than the fluid's here, stay with the rest).  The FP64 end of a
 // target's sums runs in whole warps (FP64 takes as long for 4 active lanes as
-// for 32; 32 flow channels 57 -> 41 us of a step).  On most steps no instance is due: a grid of some 30 waves strides over the targets, so
-// that such a step costs a launch and not one block per 32 targets (3-D duct,
-// 3.0M particles: 121 us, now 22).
+// for 32; 32 flow channels 57 -> 41 us of a step).  On most steps no instance is
+// due: a grid of some 30 waves strides over the targets, so that such a step
+// costs a launch and not one block per 32 targets (3-D duct, 3.0M particles:
+// 121 us, now 22).  A grid of 4 waves leaves the last one too empty (459 -> 543
+// us per step with a reinitialisation every third).
 constexpr int kReinitBlocks = 152 * 128;
 
 template <int D, int L, bool CP, bool TILE, int FORM>

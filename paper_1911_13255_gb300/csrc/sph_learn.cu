@@ -455,11 +455,11 @@ int forward(sphfsi_mpnn *m)
     launch_k(k_act, nblk(np * kC / 4, 256), 256, 0, st, (const float4 *)m->yenc, (float4 *)m->h, np * kC / 4, 0);
     for (int l = 0; l < kLayers; l++) {
         if (m->dim == 2)
-            launch_k(k_aggregate<2>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
-                                                                     m->ptr, m->idx, m->w, m->g);
+            launch_k(k_aggregate<2>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->h, (uint2 *)m->zb[l],
+                     m->n, (int)nn, m->ptr, m->idx, m->w, m->g);
         else
-            launch_k(k_aggregate<3>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->h, (uint2 *)m->zb[l], m->n, (int)nn,
-                                                                     m->ptr, m->idx, m->w, m->g);
+            launch_k(k_aggregate<3>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->h, (uint2 *)m->zb[l],
+                     m->n, (int)nn, m->ptr, m->idx, m->w, m->g);
         LTRY(gemm(m, m->zb[l], m->Wl[l], m->theta + L.b[l], m->y[l], np, kC, m->zd));
         launch_k(k_act, nblk(np * kC / 4, 256), 256, 0, st, (const float4 *)m->y[l], (float4 *)m->h, np * kC / 4, 1);
     }
@@ -489,21 +489,21 @@ int backward(sphfsi_mpnn *m, const float *dout_or_out, const float *t, const uin
              : SPHFSI_E_CUDA);
     LTRY(gemm(m, m->doutb, m->WdecT, nullptr, m->dh, np, kC, kFin));
     for (int l = kLayers - 1; l >= 0; l--) {
-        launch_k(k_dsilu, (unsigned)std::min(np / 32, 304LL), 256, 0, st, (const float4 *)m->dh, (const float4 *)m->y[l], (int)nn, (int)np,
-                                                     (uint2 *)m->dyb, m->dyT, m->grad + L.b[l]);
+        launch_k(k_dsilu, (unsigned)std::min(np / 32, 304LL), 256, 0, st, (const float4 *)m->dh,
+                 (const float4 *)m->y[l], (int)nn, (int)np, (uint2 *)m->dyb, m->dyT, m->grad + L.b[l]);
         launch_k(k_transpose, dim3((unsigned)(m->zd / 64), (unsigned)(np / 64)), 256, 0, st, m->zb[l], (int)np, m->zd,
                                                                                         m->zT);
         LTRY(gemm(m, m->dyT, m->zT, nullptr, m->grad + L.W[l], kC, m->zd, np));
         LTRY(gemm(m, m->dyb, m->WlT[l], nullptr, m->dz, np, m->zd, kC));
         if (m->dim == 2)
-            launch_k(k_agg_adjoint<2>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
-                                                                       m->ptr, m->idx, m->w, m->g);
+            launch_k(k_agg_adjoint<2>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->dz, (float4 *)m->dh,
+                     m->n, (int)nn, m->ptr, m->idx, m->w, m->g);
         else
-            launch_k(k_agg_adjoint<3>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->dz, (float4 *)m->dh, m->n, (int)nn,
-                                                                       m->ptr, m->idx, m->w, m->g);
+            launch_k(k_agg_adjoint<3>, nblk(nn, kNodes), 32 * kNodes, 0, st, (const float4 *)m->dz, (float4 *)m->dh,
+                     m->n, (int)nn, m->ptr, m->idx, m->w, m->g);
     }
-    launch_k(k_dsilu, (unsigned)std::min(np / 32, 304LL), 256, 0, st, (const float4 *)m->dh, (const float4 *)m->yenc, (int)nn, (int)np,
-                                                 (uint2 *)m->dyb, m->dyT, m->grad + L.enc_b);
+    launch_k(k_dsilu, (unsigned)std::min(np / 32, 304LL), 256, 0, st, (const float4 *)m->dh, (const float4 *)m->yenc,
+             (int)nn, (int)np, (uint2 *)m->dyb, m->dyT, m->grad + L.enc_b);
     launch_k(k_transpose, dim3(kFin / 64, (unsigned)(np / 64)), 256, 0, st, m->xb, (int)np, kFin, m->xT);
     LTRY(gemm(m, m->dyT, m->xT, nullptr, m->grad + L.enc_W, kC, kFin, np));
     return cudaGetLastError() == cudaSuccess ? SPHFSI_OK : SPHFSI_E_CUDA;

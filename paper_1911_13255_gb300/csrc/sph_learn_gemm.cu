@@ -24,8 +24,8 @@
 // 4096 x 4096 x 4096 takes 124 us (1.11 PFLOP/s; 312 us with the idle lanes of
 // warps 0 and 1 spinning next to their lane 0 and a row of 16-byte stores per
 // lane), 16384 x 256 x 4096 46 us (85), and less with a pair of CTAs (below).
-// Sharing B in clusters of 2 or 4 by
-// multicast, prefetching A into L2 and 256-byte L2 promotion change neither.
+// Sharing B in clusters of 2 or 4 by multicast, prefetching A into L2 and
+// 256-byte L2 promotion change neither.
 // Every wait is bounded; a timeout sets a status bit, skips the epilogue and
 // still frees the tensor memory.
 #include <cuda.h>   // CUtensorMap and its enums; the encoder comes from the CUDA driver library at run time
