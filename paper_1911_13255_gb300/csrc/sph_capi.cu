@@ -370,6 +370,21 @@ int request_rebuild(sphfsi_ctx *c)
     return cuda_rc(cudaMemsetAsync(c->F.held, 0xff, sizeof(int), c->st));
 }
 
+// After the device state has been replaced: the lists that follow from the
+// rows' words; and with a held configuration, a rebuild at the next step if
+// this context streams rows and the state, which came from one that did not,
+// has none.
+int rows_from_state(sphfsi_ctx *c)
+{
+    if (c->F.n == 0) return SPHFSI_OK;
+    TRY(launch_row_parts(c->F, c->st));
+    if (!c->F.list || !held_on(c->F)) return SPHFSI_OK;
+    uint32_t word = 0;
+    TRY(cuda_rc(cudaMemcpyAsync(&word, c->F.nbc, sizeof(word), cudaMemcpyDeviceToHost, c->st)));
+    TRY(cuda_rc(cudaStreamSynchronize(c->st)));
+    return word ? SPHFSI_OK : request_rebuild(c);
+}
+
 int check_ctx(sphfsi_ctx *c, bool need_final)
 {
     if (!c) return SPHFSI_E_INVAL;
@@ -1912,7 +1927,7 @@ int sphfsi_set_state(sphfsi_ctx *c, const void *blob, int64_t bytes)
     c->failed = fail == kFailWait;
     c->runaway = fail == kFailRunaway;
     c->last_status = 0;
-    return SPHFSI_OK;
+    return rows_from_state(c);
 }
 
 int sphfsi_get_info(sphfsi_ctx *c, sphfsi_info *out)
@@ -2050,6 +2065,8 @@ int sphfsi_set_tuning(sphfsi_ctx *c, const sphfsi_tuning *t)
     c->F.split_records = t->records == 1 ? 1 : 0;
     c->F.bin_fused = t->records == 2 ? 1 : 0;
     c->F.rows = t->rows;
+    // a held configuration built without rows has none to stream
+    if (t->list && !c->F.list && held_on(c->F)) TRY(request_rebuild(c));
     c->F.list = t->list;
     if (t->list_lanes) c->F.list_lanes = t->list_lanes;
     c->S.force_lane_path = t->solid_variant;
@@ -2082,7 +2099,9 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
     TRY(check_ctx(c, true));
     if (!best || steps < 1 || steps > 10000 || std::isnan(dt_F) || c->st == nullptr) return SPHFSI_E_INVAL;
     TRY(cuda_rc(cudaStreamSynchronize(c->st)));
-    // snapshot of every device allocation, restored before each trial and at the end
+    sphfsi_tuning cur{}, keep{};
+    sphfsi_get_tuning(c, &keep);
+    // snapshot of every device allocation of the state, restored before each trial and at the end
     size_t total = 0;
     for (auto &a : c->allocs) total += (a.second + 255) & ~(size_t)255;
     char *snap = nullptr;
@@ -2098,11 +2117,13 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
             if (cudaMemcpyAsync(dst, src, a.second, cudaMemcpyDeviceToDevice, c->st) != cudaSuccess) return SPHFSI_E_CUDA;
             off += (a.second + 255) & ~(size_t)255;
         }
+        if (!save) {
+            c->F.list = keep.list;   // the restored rows are the ones of the snapshot's form
+            TRY(rows_from_state(c));
+        }
         return cuda_rc(cudaStreamSynchronize(c->st));
     };
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    sphfsi_tuning cur{}, keep{};
-    sphfsi_get_tuning(c, &keep);
     int rc = copy_all(true);
     if (!rc) rc = cuda_rc(cudaEventCreate(&e0));
     if (!rc) rc = cuda_rc(cudaEventCreate(&e1));

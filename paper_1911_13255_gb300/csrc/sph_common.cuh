@@ -216,7 +216,9 @@ struct Fluid {
     uint32_t *nbc;
     // targets that the row build lists apart: [kPartNear] those with solid
     // particles in their neighbour cells and overflowed rows, [kPartWall]
-    // those with wall neighbours and no solid particles
+    // those with wall neighbours and no solid particles.  They hold as long as
+    // nbc and follow from it: no part of a checkpoint, made again from the
+    // restored nbc (launch_row_parts)
     int *part[2];
     int *part_n;
     float4 *B4;           // boundary part of a target's density rate: coefficient on v^{n+1}, constant
@@ -224,8 +226,10 @@ struct Fluid {
 
 // nbc flags: solid particles in one of the target's neighbour cells (the pair
 // loops visit those cells for the solid candidates); the row overflowed (the
-// target takes the cell visit for everything)
-constexpr uint32_t kListSolid = 1u << 22, kListOver = 1u << 23;
+// target takes the cell visit for everything); the word is a built row's (a
+// rebuild step without rows clears slot 0's word, so nbc[0] == 0 says that the
+// rows are not those of the current pair configuration)
+constexpr uint32_t kListSolid = 1u << 22, kListOver = 1u << 23, kListBuilt = 1u << 24;
 constexpr uint32_t kListCountMask = 0x7ffu;
 constexpr uint32_t kListWalls = kListCountMask << 11;   // nW != 0
 enum : int { kPartNear = 0, kPartWall = 1 };
@@ -481,6 +485,8 @@ int launch_solid_fluid_force(const Batch &bt, const Fluid &f, const Solid &s, in
 int launch_density(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int dim, cudaStream_t st);
 // neighbour rows of the fluid targets (Fluid::list), on rebuild steps
 int launch_pairlist(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int dim, cudaStream_t st);
+// the lists of targets apart (Fluid::part) from the rows' words
+int launch_row_parts(const Fluid &f, cudaStream_t st);
 int launch_debug_pairs(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int dim, int inst,
                        int which, int *counts, int *offs, int *out, cudaStream_t st);
 

@@ -184,14 +184,12 @@ int launch_momentum(const Batch &bt, const Fluid &f, const Walls &w, const Solid
 // target then takes the cell form; every write stays inside the row).  Runs on
 // rebuild steps.
 // ---------------------------------------------------------------------------
-// Row i's word; a row with boundary neighbours, or one that overflowed, also
-// enters the list of its kind, one atomic per warp and kind (the order of a
+// Row i's word (row_word); a row with boundary neighbours, or one that
+// overflowed, also enters the list of its kind (row_part), one atomic per warp and kind (the order of a
 // list does not matter: every target is summed by its own lanes).
-__device__ __forceinline__ void row_word(const Fluid &f, int i, int nF, int nW, bool solid)
+__device__ __forceinline__ void row_part(const Fluid &f, int i, uint32_t word)
 {
-    const bool over = nF + nW > f.list_cap || nF > (int)kListCountMask || nW > (int)kListCountMask;
-    f.nbc[i] = over ? kListOver : ((uint32_t)nF | ((uint32_t)nW << 11) | (solid ? kListSolid : 0u));
-    const int kind = solid || over ? kPartNear : (nW ? kPartWall : -1);
+    const int kind = word & (kListSolid | kListOver) ? kPartNear : (word & kListWalls ? kPartWall : -1);
     const unsigned here = __activemask();
     const int lane = threadIdx.x & 31;
     for (int p = 0; p < 2; p++) {
@@ -203,6 +201,29 @@ __device__ __forceinline__ void row_word(const Fluid &f, int i, int nF, int nW, 
         base = __shfl_sync(m, base, lead);
         f.part[p][base + __popc(m & ((1u << lane) - 1u))] = i;
     }
+}
+__device__ __forceinline__ void row_word(const Fluid &f, int i, int nF, int nW, bool solid)
+{
+    const bool over = nF + nW > f.list_cap || nF > (int)kListCountMask || nW > (int)kListCountMask;
+    const uint32_t word =
+        kListBuilt | (over ? kListOver : ((uint32_t)nF | ((uint32_t)nW << 11) | (solid ? kListSolid : 0u)));
+    f.nbc[i] = word;
+    row_part(f, i, word);
+}
+
+// The lists again from words that came from elsewhere (a restored state).
+__global__ void k_row_parts(Fluid f)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < f.n) row_part(f, i, f.nbc[i]);
+}
+
+int launch_row_parts(const Fluid &f, cudaStream_t st)
+{
+    if (f.n == 0) return 0;
+    if (cudaMemsetAsync(f.part_n, 0, 2 * sizeof(int), st) != cudaSuccess) return -3;
+    k_row_parts<<<(f.n + 255) / 256, 256, 0, st>>>(f);
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 // One warp per cell, in two stages:
