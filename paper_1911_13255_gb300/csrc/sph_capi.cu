@@ -370,12 +370,15 @@ int request_rebuild(sphfsi_ctx *c)
     return cuda_rc(cudaMemsetAsync(c->F.held, 0xff, sizeof(int), c->st));
 }
 
-// After the device state has been replaced: the lists that follow from the
-// rows' words; and with a held configuration, a rebuild at the next step if
-// this context streams rows and the state, which came from one that did not,
-// has none.
-int rows_from_state(sphfsi_ctx *c)
+// After the device state has been replaced, what lives beside it: equal phase
+// counts for the CTAs of the windowed sub-step kernel (a time-out leaves them
+// unequal); the lists that follow from the rows' words; and with a held
+// configuration, a rebuild at the next step if this context streams rows and
+// the state, which came from one that did not, has none.
+int scratch_from_state(sphfsi_ctx *c)
 {
+    if (c->S.win_ctas)
+        TRY(cuda_rc(cudaMemsetAsync(c->S.win_flag, 0, sizeof(unsigned) * 32 * (size_t)c->S.win_ctas, c->st)));
     if (c->F.n == 0) return SPHFSI_OK;
     TRY(launch_row_parts(c->F, c->st));
     if (!c->F.list || !held_on(c->F)) return SPHFSI_OK;
@@ -1917,9 +1920,6 @@ int sphfsi_set_state(sphfsi_ctx *c, const void *blob, int64_t bytes)
         TRY(cuda_rc(cudaMemcpy(a.first, p, a.second, cudaMemcpyHostToDevice)));
         p += a.second;
     }
-    // after a time-out the CTAs of the windowed kernel may have published
-    // different numbers of phases
-    if (c->S.win_ctas) TRY(cuda_rc(cudaMemset(c->S.win_flag, 0, sizeof(unsigned) * 32 * (size_t)c->S.win_ctas)));
     // steps are allowed again unless the checkpoint itself was taken after a
     // scan that gave up or a step that ran away
     int fail = 0;
@@ -1927,7 +1927,7 @@ int sphfsi_set_state(sphfsi_ctx *c, const void *blob, int64_t bytes)
     c->failed = fail == kFailWait;
     c->runaway = fail == kFailRunaway;
     c->last_status = 0;
-    return rows_from_state(c);
+    return scratch_from_state(c);
 }
 
 int sphfsi_get_info(sphfsi_ctx *c, sphfsi_info *out)
@@ -2119,7 +2119,7 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
         }
         if (!save) {
             c->F.list = keep.list;   // the restored rows are the ones of the snapshot's form
-            TRY(rows_from_state(c));
+            TRY(scratch_from_state(c));
         }
         return cuda_rc(cudaStreamSynchronize(c->st));
     };

@@ -326,8 +326,9 @@ struct Batch {
     int B;
     int ncell;                    // total cells
     long long spin;               // iterations of a bounded wait before it gives up (sphfsi_set_wait_limit)
-    // Stops the context's device work: kFailWait when the histogram scan gave
-    // up waiting (the cell starts of the step are then not valid, so every
+    // Stops the context's device work: kFailWait when a bounded wait of a step
+    // gave up (set by the finish kernel) or, at once, when the histogram scan
+    // gave up (the cell starts of the step are then not valid, so every
     // later kernel that reads cell ranges returns at once), kFailRunaway when
     // a step ended with a non-finite or run-away state (the finish kernel sets
     // it; the next step's kernels return at once, so a blown-up state never

@@ -170,6 +170,11 @@ __global__ void k_finish(Batch bt, int learned, unsigned *gbar, Fluid f)
     // has run away, and the context's later steps do nothing
     if (!(vF <= 3.0e38f) || !(vS <= 3.0e38f) || !(aS <= 3.0e38f) || vF > bt.I[b].P.c0)
         ctl->status |= ST_NONFINITE;
+    // a wait that gave up in this step (the solid branch has joined): the steps
+    // already queued behind it do nothing either.  They would compute from a
+    // half-finished state, and the windowed sub-step kernel's CTAs, which have
+    // published unequal numbers of phases, would wait out the limit in each.
+    if (ctl->status & ST_TIMEOUT) atomicCAS(bt.fail, 0, kFailWait);
     if (ctl->status & ST_NONFINITE) atomicCAS(bt.fail, 0, kFailRunaway);
     // the maxima of this step set the next step's dt_F and K
     ctl->prev_vmaxF = vF;
