@@ -36,7 +36,9 @@
  *   - Array arguments may be host pointers or CUDA device pointers (unified
  *     addressing decides); the caller owns them; the library copies.
  *   - All work is issued on the stream given to sphfsi_create; getters and
- *     sphfsi_sync wait for it.
+ *     sphfsi_sync wait for it.  A getter that waits also comes after what is
+ *     queued on the legacy default stream when it writes to device or pinned
+ *     memory.
  *   - A context is used by one host thread at a time.
  */
 #ifndef SPHFSI_H

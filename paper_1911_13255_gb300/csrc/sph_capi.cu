@@ -155,6 +155,7 @@ struct sphfsi_ctx {
     // side stream for the solid branch, which runs beside momentum and continuity
     cudaStream_t side = nullptr;
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+    cudaEvent_t read_ev = nullptr;   // the default stream's position at a read
     // asynchronous read of the solid positions: each device slot's output
     // row (original order), and the gathered rows
     int *d_orow = nullptr;
@@ -703,15 +704,33 @@ struct Output {
 // new arrays 15 ms, 1 ms of it left when the host touches them first).  So the
 // host does, with all its threads where that pays for starting them; the copy
 // overwrites the bytes.
-// (callers pass pointers of any kind)
-bool plain_host(const void *p)
+// (callers pass pointers of any kind; memory that the device reaches too may
+// have work of the caller's queued on it, so the host touches pageable memory
+// only)
+cudaMemoryType memory_kind(const void *p)
 {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return cudaMemoryTypeManaged;
     }
-    return at.type == cudaMemoryTypeUnregistered || at.type == cudaMemoryTypeHost;
+    return at.type;
+}
+bool pageable(const void *p) { return memory_kind(p) == cudaMemoryTypeUnregistered; }
+bool plain_host(const void *p)
+{
+    const cudaMemoryType t = memory_kind(p);
+    return t == cudaMemoryTypeUnregistered || t == cudaMemoryTypeHost;
+}
+
+// Work that the caller has queued on the default stream may still write or read
+// an output in memory that the device reaches: the context's stream, which
+// need not wait for that one by itself, goes behind it.
+int after_default_stream(sphfsi_ctx *c)
+{
+    if (c->st == nullptr) return SPHFSI_OK;
+    TRY(cuda_rc(cudaEventRecord(c->read_ev, cudaStreamLegacy)));
+    return cuda_rc(cudaStreamWaitEvent(c->st, c->read_ev, 0));
 }
 
 void touch_pages(const std::vector<Output> &outs)
@@ -719,7 +738,7 @@ void touch_pages(const std::vector<Output> &outs)
     const long os = sysconf(_SC_PAGESIZE);
     const size_t page = os > 0 ? (size_t)os : 4096, threads_from = (size_t)16 << 20;
     for (const Output &o : outs) {
-        if (!o.dst || !plain_host(o.dst)) continue;
+        if (!o.dst || !pageable(o.dst)) continue;
         volatile char *p = (volatile char *)o.dst;
         const int64_t pages = (int64_t)((o.bytes + page - 1) / page);
         host_parallel(pages, o.bytes < threads_from ? 1 : host_chunks(pages, 64), [&](int, int64_t lo, int64_t hi) {
@@ -763,8 +782,13 @@ int read_rows(sphfsi_ctx *c, std::vector<Output> outs, Fill &&fill)
     };
     const bool together = room(total);
     if (!together && !room(most)) return SPHFSI_E_NOMEM;
-    bool one_copy = total <= kOneCopy && together;
-    for (const Output &o : outs) one_copy = one_copy && (!o.dst || plain_host(o.dst));
+    bool one_copy = total <= kOneCopy && together, shared = false;
+    for (const Output &o : outs)
+        if (o.dst) {
+            one_copy = one_copy && plain_host(o.dst);
+            shared = shared || !pageable(o.dst);
+        }
+    if (shared) TRY(after_default_stream(c));
     if (one_copy) {
         size_t off = 0;
         for (Output &o : outs) {
@@ -1482,6 +1506,7 @@ int sphfsi_finalize(sphfsi_ctx *c)
     }
     TRY(cuda_rc(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming)));
     TRY(cuda_rc(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming)));
+    TRY(cuda_rc(cudaEventCreateWithFlags(&c->read_ev, cudaEventDisableTiming)));
     c->finalized = true;
     // release the host staging copies that are not needed any more
     for (auto &h : c->ih) {
@@ -1673,6 +1698,8 @@ int sphfsi_get_solid_positions_async(sphfsi_ctx *c, double *r)
 
 int sphfsi_get_solid_positions_all(sphfsi_ctx *c, double *r)
 {
+    TRY(check_ctx(c, true));
+    if (r && !pageable(r)) TRY(after_default_stream(c));
     TRY(sphfsi_get_solid_positions_async(c, r));
     return cuda_rc(cudaStreamSynchronize(c->st));
 }
@@ -2418,6 +2445,7 @@ void sphfsi_destroy(sphfsi_ctx *c)
         if (c->ev[k]) cudaEventDestroy(c->ev[k]);
     if (c->fork_ev) cudaEventDestroy(c->fork_ev);
     if (c->join_ev) cudaEventDestroy(c->join_ev);
+    if (c->read_ev) cudaEventDestroy(c->read_ev);
     if (c->side) cudaStreamDestroy(c->side);
     for (auto &a : c->allocs) cudaFree(a.first);
     for (void *p : c->scratch) cudaFree(p);
