@@ -38,7 +38,10 @@
  *   - All work is issued on the stream given to sphfsi_create; getters and
  *     sphfsi_sync wait for it.  A getter that waits also comes after what is
  *     queued on the legacy default stream when it writes to device or pinned
- *     memory.
+ *     memory.  The state getters stage rows in device memory: 1 MB that a
+ *     context always holds, and from the first larger read on a buffer of that
+ *     read's size, at most 64 MB, kept until sphfsi_destroy (a read for which
+ *     there is no more device memory makes do with the 1 MB).
  *   - A context is used by one host thread at a time.
  */
 #ifndef SPHFSI_H

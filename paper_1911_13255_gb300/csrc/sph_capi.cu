@@ -160,7 +160,9 @@ struct sphfsi_ctx {
     // row (original order), and the gathered rows
     int *d_orow = nullptr;
     double *d_spos = nullptr;
-    // staging buffer of the state reads, grown on demand
+    // staging of the state reads: kOneCopy bytes, and a larger buffer from the
+    // first larger read on
+    uint8_t *d_read0 = nullptr;
     void *d_read = nullptr;
     size_t read_bytes = 0;
     std::vector<uint8_t> h_read;   // at most kOneCopy bytes
@@ -695,8 +697,8 @@ namespace {
 
 struct Output {
     void *dst;      // caller's pointer (host or device), null: not asked for
-    size_t bytes;
-    void *dev;      // its rows on the device
+    size_t row;     // bytes per row
+    void *dev;      // its staged rows on the device
 };
 
 // Pages of a fresh host array are mapped at their first touch: 3 us each from
@@ -733,105 +735,115 @@ int after_default_stream(sphfsi_ctx *c)
     return cuda_rc(cudaStreamWaitEvent(c->st, c->read_ev, 0));
 }
 
-void touch_pages(const std::vector<Output> &outs)
+void touch_pages(const std::vector<Output> &outs, size_t n)
 {
     const long os = sysconf(_SC_PAGESIZE);
     const size_t page = os > 0 ? (size_t)os : 4096, threads_from = (size_t)16 << 20;
     for (const Output &o : outs) {
         if (!o.dst || !pageable(o.dst)) continue;
         volatile char *p = (volatile char *)o.dst;
-        const int64_t pages = (int64_t)((o.bytes + page - 1) / page);
-        host_parallel(pages, o.bytes < threads_from ? 1 : host_chunks(pages, 64), [&](int, int64_t lo, int64_t hi) {
+        const size_t bytes = n * o.row;
+        const int64_t pages = (int64_t)((bytes + page - 1) / page);
+        host_parallel(pages, bytes < threads_from ? 1 : host_chunks(pages, 64), [&](int, int64_t lo, int64_t hi) {
             for (int64_t k = lo; k < hi; k++) p[(size_t)k * page] = 0;
         });
     }
 }
 
-constexpr size_t kOneCopy = (size_t)1 << 20;
+// Staging of the rows on the device: up to kOneCopy bytes in a buffer that
+// every context has from the start, more in one that grows with the first
+// larger read and stays, up to kReadMost bytes; a state beyond that, or one
+// whose larger buffer the device has no memory for, goes out in ranges of
+// rows (one pass over the slots each, 10 us on 3.0M particles).
+constexpr size_t kOneCopy = (size_t)1 << 20, kReadMost = (size_t)64 << 20;
 
-// fill(outs) enqueues the kernel that writes every asked-for output's rows to
-// its dev pointer.  All outputs are staged together in one buffer that the
-// context keeps for the next read; where it cannot have that much device
-// memory, one after the other.
+// fill(outs, row0, rows) enqueues the kernel that writes rows [row0, row0 +
+// rows) of every asked-for output to its dev pointer.
 template <typename Fill>
-int read_rows(sphfsi_ctx *c, std::vector<Output> outs, Fill &&fill)
+int read_rows(sphfsi_ctx *c, int n, std::vector<Output> outs, Fill &&fill)
 {
-    auto padded = [](size_t n) { return (n + 255) & ~(size_t)255; };
-    size_t total = 0, most = 0;
-    for (const Output &o : outs)
-        if (o.dst) {
-            total += padded(o.bytes);
-            most = std::max(most, padded(o.bytes));
-        }
-    if (total == 0) return cuda_rc(cudaStreamSynchronize(c->st));
-    auto room = [&](size_t need) {
-        if (need <= c->read_bytes) return true;
-        if (c->d_read) {
-            cudaStreamSynchronize(c->st);
-            cudaFree(c->d_read);
-        }
-        c->d_read = nullptr;
-        c->read_bytes = 0;
-        if (cudaMalloc(&c->d_read, need) != cudaSuccess) {
-            cudaGetLastError();
-            c->d_read = nullptr;
-            return false;
-        }
-        c->read_bytes = need;
-        return true;
+    auto padded = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    auto staged = [&](size_t rows) {
+        size_t b = 0;
+        for (const Output &o : outs) b += o.dst ? padded(rows * o.row) : 0;
+        return b;
     };
-    const bool together = room(total);
-    if (!together && !room(most)) return SPHFSI_E_NOMEM;
-    bool one_copy = total <= kOneCopy && together, shared = false;
+    const size_t total = staged((size_t)n);
+    if (total == 0) return cuda_rc(cudaStreamSynchronize(c->st));
+    uint8_t *buf = (uint8_t *)c->d_read0;
+    size_t size = kOneCopy;
+    if (total > kOneCopy) {
+        const size_t want = std::min(total, kReadMost);
+        if (c->read_bytes < want) {
+            if (c->d_read) {
+                cudaStreamSynchronize(c->st);
+                cudaFree(c->d_read);
+            }
+            c->d_read = nullptr;
+            c->read_bytes = 0;
+            if (cudaMalloc(&c->d_read, want) == cudaSuccess) {
+                c->read_bytes = want;
+            } else {
+                cudaGetLastError();
+                c->d_read = nullptr;
+            }
+        }
+        if (c->d_read) {
+            buf = (uint8_t *)c->d_read;
+            size = c->read_bytes;
+        }
+    }
+    bool one_copy = total <= kOneCopy, shared = false;
     for (const Output &o : outs)
         if (o.dst) {
             one_copy = one_copy && plain_host(o.dst);
             shared = shared || !pageable(o.dst);
         }
     if (shared) TRY(after_default_stream(c));
-    if (one_copy) {
+    if (!one_copy) touch_pages(outs, (size_t)n);
+    // (the rows' padding: 256 bytes an output at most)
+    size_t row = 0, many = 0;
+    for (const Output &o : outs)
+        if (o.dst) {
+            row += o.row;
+            many++;
+        }
+    const int64_t most = staged((size_t)n) <= size ? n : (int64_t)((size - 256 * many) / row);
+    for (int64_t r0 = 0; r0 < n; r0 += most) {
+        const size_t rows = (size_t)std::min(most, (int64_t)n - r0);
         size_t off = 0;
         for (Output &o : outs) {
-            o.dev = o.dst ? (uint8_t *)c->d_read + off : nullptr;
-            if (o.dst) off += padded(o.bytes);
+            o.dev = o.dst ? buf + off : nullptr;
+            if (o.dst) off += padded(rows * o.row);
         }
-        fill(outs);
+        fill(outs, (int)r0, (int)rows);
         TRY(cuda_rc(cudaGetLastError()));
-        std::vector<uint8_t> &rows = c->h_read;   // kept: its pages are mapped once
-        if (rows.size() < total) rows.resize(total);
-        TRY(cuda_rc(cudaMemcpyAsync(rows.data(), c->d_read, total, cudaMemcpyDeviceToHost, c->st)));
-        TRY(cuda_rc(cudaStreamSynchronize(c->st)));
+        if (one_copy) {
+            std::vector<uint8_t> &h = c->h_read;   // kept: its pages are mapped once
+            if (h.size() < total) h.resize(total);
+            TRY(cuda_rc(cudaMemcpyAsync(h.data(), buf, total, cudaMemcpyDeviceToHost, c->st)));
+            TRY(cuda_rc(cudaStreamSynchronize(c->st)));
+            for (const Output &o : outs)
+                if (o.dst) std::memcpy(o.dst, h.data() + ((uint8_t *)o.dev - buf), rows * o.row);
+            return SPHFSI_OK;
+        }
         for (const Output &o : outs)
-            if (o.dst) std::memcpy(o.dst, rows.data() + ((uint8_t *)o.dev - (uint8_t *)c->d_read), o.bytes);
-        return SPHFSI_OK;
-    }
-    touch_pages(outs);
-    for (size_t k = 0; k < outs.size(); k++) {
-        std::vector<Output> now(outs);
-        size_t off = 0;
-        for (size_t j = 0; j < now.size(); j++) {
-            if (!together && j != k) now[j].dst = nullptr;
-            now[j].dev = now[j].dst ? (uint8_t *)c->d_read + off : nullptr;
-            if (now[j].dst) off += padded(now[j].bytes);
-        }
-        if (off == 0) continue;
-        fill(now);
-        TRY(cuda_rc(cudaGetLastError()));
-        for (const Output &o : now)
-            if (o.dst) TRY(cuda_rc(cudaMemcpyAsync(o.dst, o.dev, o.bytes, cudaMemcpyDefault, c->st)));
-        if (together) break;
+            if (o.dst)
+                TRY(cuda_rc(cudaMemcpyAsync((uint8_t *)o.dst + (size_t)r0 * o.row, o.dev, rows * o.row,
+                                            cudaMemcpyDefault, c->st)));
     }
     return cuda_rc(cudaStreamSynchronize(c->st));
 }
 
-// rows of n slots of the fluid state (the pointers at the instance's first slot)
+// rows [row0, row0 + rows) of the fluid state of the n slots from f0
 template <int D>
-__global__ void k_read_fluid(FluidState S, const float *dvdt, int f0, int n, double rho0, double *r, float *v,
-                             double *rho, float *rate, float *acc)
+__global__ void k_read_fluid(FluidState S, const float *dvdt, int f0, int n, int row0, int rows, double rho0, double *r,
+                             float *v, double *rho, float *rate, float *acc)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
-    const int k = f0 + t, i = S.id[k];
+    const int k = f0 + t, i = S.id[k] - row0;
+    if ((unsigned)i >= (unsigned)rows) return;
     if (r) {
         r[(size_t)i * D] = S.x[k];
         r[(size_t)i * D + 1] = S.y[k];
@@ -850,13 +862,15 @@ __global__ void k_read_fluid(FluidState S, const float *dvdt, int f0, int n, dou
 
 // orow: a slot's row among all instances' (original order)
 template <int D>
-__global__ void k_read_solid(Solid S, const int *orow, int s0, int n, double *r, float *v, double *F, double *vbar,
+__global__ void k_read_solid(Solid S, const int *orow, int s0, int n, int row0, int rows, double *r, float *v, double *F, double *vbar,
                              double *abar, float *fF, float *nrm)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     const int k = s0 + t;
-    const size_t o = (size_t)(orow[k] - s0) * D;
+    const int i = orow[k] - s0 - row0;
+    if ((unsigned)i >= (unsigned)rows) return;
+    const size_t o = (size_t)i * D;
     if (r) {
         r[o] = S.x[k];
         r[o + 1] = S.y[k];
@@ -869,8 +883,8 @@ __global__ void k_read_solid(Solid S, const int *orow, int s0, int n, double *r,
         if (D == 3) v[o + 2] = u.z;
     }
     if (F)
-        for (int i = 0; i < D * D; i++)
-            F[o * D + i] = (double)S.H[9 * (size_t)k + i] + ((i % (D + 1)) == 0 ? 1.0 : 0.0);
+        for (int m = 0; m < D * D; m++)
+            F[o * D + m] = (double)S.H[9 * (size_t)k + m] + ((m % (D + 1)) == 0 ? 1.0 : 0.0);
     for (int q = 0; q < D; q++) {
         if (vbar) vbar[o + q] = S.vbar[3 * (size_t)k + q];
         if (abar) abar[o + q] = S.abar[3 * (size_t)k + q];
@@ -1230,6 +1244,7 @@ int sphfsi_finalize(sphfsi_ctx *c)
     }
     TRY(dalloc(c, &F.bsum, 4096));
     TRY(dalloc(c, &F.gbar, 2));
+    TRY(dscratch(c, &c->d_read0, kOneCopy));
     // neighbour rows (tuned): about 20 (2-D) or 80 (3-D) neighbours per fluid
     // particle on a lattice, wall neighbours included.  On from 32 768 fluid
     // particles in 2-D (2 lanes per target) and 16 384 in 3-D (4).  Step with the
@@ -1630,16 +1645,16 @@ int sphfsi_get_fluid(sphfsi_ctx *c, double *r, float *v, double *rho, float *drh
     const InstHost &h = c->ih[c->sel];
     const int n = (int)h.nf, f0 = h.d.f0;
     if (n == 0) return cuda_rc(cudaStreamSynchronize(c->st));
-    const size_t nd = (size_t)n * D;
-    return read_rows(c,
-                     {{r, nd * sizeof(double), nullptr},
-                      {v, nd * sizeof(float), nullptr},
-                      {rho, n * sizeof(double), nullptr},
-                      {drho_dt, n * sizeof(float), nullptr},
-                      {dvdt, nd * sizeof(float), nullptr}},
-                     [&](const std::vector<Output> &o) {
+    const size_t vd = D * sizeof(double), vf = D * sizeof(float);
+    return read_rows(c, n,
+                     {{r, vd, nullptr},
+                      {v, vf, nullptr},
+                      {rho, sizeof(double), nullptr},
+                      {drho_dt, sizeof(float), nullptr},
+                      {dvdt, vf, nullptr}},
+                     [&](const std::vector<Output> &o, int row0, int rows) {
                          auto kern = D == 3 ? k_read_fluid<3> : k_read_fluid<2>;
-                         kern<<<(n + 255) / 256, 256, 0, c->st>>>(c->F.s[0], c->F.dvdt, f0, n, h.f_rho0,
+                         kern<<<(n + 255) / 256, 256, 0, c->st>>>(c->F.s[0], c->F.dvdt, f0, n, row0, rows, h.f_rho0,
                                                                   (double *)o[0].dev, (float *)o[1].dev,
                                                                   (double *)o[2].dev, (float *)o[3].dev,
                                                                   (float *)o[4].dev);
@@ -1653,21 +1668,22 @@ int sphfsi_get_solid(sphfsi_ctx *c, double *r, float *v, double *F, double *vbar
     const InstHost &h = c->ih[c->sel];
     const int n = (int)h.ns, s0 = h.d.s0;
     if (n == 0) return cuda_rc(cudaStreamSynchronize(c->st));
-    const size_t nd = (size_t)n * D;
-    return read_rows(c,
-                     {{r, nd * sizeof(double), nullptr},
-                      {v, nd * sizeof(float), nullptr},
-                      {F, nd * D * sizeof(double), nullptr},
-                      {vbar, nd * sizeof(double), nullptr},
-                      {abar, nd * sizeof(double), nullptr},
-                      {fF, nd * sizeof(float), nullptr},
-                      {nrm, nd * sizeof(float), nullptr}},
-                     [&](const std::vector<Output> &o) {
+    const size_t vd = D * sizeof(double), vf = D * sizeof(float);
+    return read_rows(c, n,
+                     {{r, vd, nullptr},
+                      {v, vf, nullptr},
+                      {F, vd * D, nullptr},
+                      {vbar, vd, nullptr},
+                      {abar, vd, nullptr},
+                      {fF, vf, nullptr},
+                      {nrm, vf, nullptr}},
+                     [&](const std::vector<Output> &o, int row0, int rows) {
                          auto kern = D == 3 ? k_read_solid<3> : k_read_solid<2>;
-                         kern<<<(n + 127) / 128, 128, 0, c->st>>>(c->S, c->d_orow, s0, n, (double *)o[0].dev,
-                                                                  (float *)o[1].dev, (double *)o[2].dev,
-                                                                  (double *)o[3].dev, (double *)o[4].dev,
-                                                                  (float *)o[5].dev, (float *)o[6].dev);
+                         kern<<<(n + 127) / 128, 128, 0, c->st>>>(c->S, c->d_orow, s0, n, row0, rows,
+                                                                  (double *)o[0].dev, (float *)o[1].dev,
+                                                                  (double *)o[2].dev, (double *)o[3].dev,
+                                                                  (double *)o[4].dev, (float *)o[5].dev,
+                                                                  (float *)o[6].dev);
                      });
 }
 
