@@ -37,7 +37,7 @@ __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, con
                                 [&](int j) { return f.W4[j]; },
                                 [&](int, const float4 &, const float4 &Wj, const float *d, float r2, float, float,
                                     float) {
-                if (!(r2 >= kMinNormal)) return;   // a clumped pair: no direction, dW(0) = 0
+                if (r2 < kMinNormal) return;   // a clumped pair: no direction, dW(0) = 0 (a NaN goes through)
                 const float rhoj = P.rho0 + Wj.w;
                 const float r = r2 * rsqrt_normal(r2), a = 1.0f - half_inv_h * r;
                 const float dot = (vi[0] - Wj.x) * d[0] + (vi[1] - Wj.y) * d[1] +

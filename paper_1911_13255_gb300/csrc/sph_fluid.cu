@@ -70,8 +70,9 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
                                       [&](int, const float4 &Pj, const float4 &Vj, const float *d, float r2, float,
                                           float, float) {
                 // two particles at one FP32 position (a clumped pair): the
-                // direction is undefined and the pair's terms vanish with r
-                if (!(r2 >= kMinNormal)) return;
+                // direction is undefined and the pair's terms vanish with r (a NaN
+                // goes through, into the sums)
+                if (r2 < kMinNormal) return;
                 const float rhoj = P.rho0 + Vj.w;
                 const float invr = rsqrt_normal(r2);
                 const float a = 1.0f - half_inv_h * (r2 * invr);
@@ -108,6 +109,9 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
         f.W4[i] = make_float4(vn[0], vn[1], vn[2], Vi.w);
         if (SETS != kFluidOnly) f.B4[i] = make_float4(bnd[0], bnd[1], bnd[2], bnd[3]);
         cnt.vmax = sqrtf(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
+        // a position that is no number is in nobody's support where rows or
+        // compacted lists are tested with "<": the finish kernel hears of it here
+        if (Pi.x != Pi.x || Pi.y != Pi.y || (D == 3 && Pi.z != Pi.z)) cnt.vmax = __int_as_float(0x7fffffff);
         if (SETS == kAllSets) {
             float Vi_ = P.mF / rhoi;   // force = V_i * afs (same V_i as the solid side)
             for (int k = 0; k < D; k++) cnt.mom[k] = (double)(Vi_ * afs[k]);
