@@ -151,6 +151,7 @@ struct sphfsi_ctx {
     cudaEvent_t ev[kEvents] = {};
     int kernels_per_step = 0;
     bool fork_first = false;   // the solid branch starts before the neighbour rows are built
+    bool two_forms = false;    // some instances take rows, some the cell form (until the tuning is set)
     int max_reach = 1;   // largest cell reach of the instances (sphfsi_params::cell_reach)
     // side stream for the solid branch, which runs beside momentum and continuity
     cudaStream_t side = nullptr;
@@ -329,11 +330,17 @@ int enqueue_step(sphfsi_ctx *c, double dt)
     // is the longer one (fork_first) the rows wait until it has started: the
     // reinitialisation, which it waits for, then visits the cells.
     const bool late_rows = c->F.list && c->fork_first && c->S.n;
-    Fluid cells = c->F;
-    if (late_rows) cell_form(c, cells);
-    else TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
+    Fluid rows = c->F, cells = c->F;
+    if (late_rows || c->two_forms) cell_form(c, cells);
+    if (c->two_forms) rows.only = 1, cells.only = 0;
+    auto pair_loop = [&](auto launch) -> int {
+        if (c->two_forms) TRY(launch(c->bt, cells, c->W, c->S, D, st));
+        return launch(c->bt, rows, c->W, c->S, D, st);
+    };
+    if (!late_rows) TRY(launch_pairlist(c->bt, rows, c->W, c->S, D, st));
     TRY(mark(c, 1));
-    TRY(launch_reinit(c->bt, late_rows ? cells : c->F, c->W, c->S, D, st));
+    if (late_rows) TRY(launch_reinit(c->bt, cells, c->W, c->S, D, st));
+    else TRY(pair_loop(launch_reinit));
     TRY(mark(c, 3));
     // The solid branch (a5, then a7 + a8) depends only on the records written
     // so far, so it runs on the side stream while the main stream does a4
@@ -354,15 +361,16 @@ int enqueue_step(sphfsi_ctx *c, double dt)
         TRY(cuda_rc(cudaEventRecord(c->join_ev, c->side)));
     }
     if (late_rows) TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
-    TRY(launch_momentum(c->bt, c->F, c->W, c->S, D, st));
+    TRY(pair_loop(launch_momentum));
     TRY(mark(c, 5));
-    TRY(launch_density(c->bt, c->F, c->W, c->S, D, st));
+    TRY(pair_loop(launch_density));
     TRY(mark(c, 6));
     if (c->S.n) TRY(cuda_rc(cudaStreamWaitEvent(st, c->join_ev, 0)));
     TRY(launch_finish(c->bt, c->S.learned, c->F.gbar, c->F, st));
     TRY(mark(c, 9));
     // kernels of this library per step (memsets excluded)
     c->kernels_per_step = 4 + bin_kernels(c->F) + (c->S.n ? 2 : 0) + (c->F.list && c->F.n ? 1 : 0) +
+                          (c->two_forms ? 3 : 0) +
                           (c->S.learned ? 5 + mpnn_kernels_per_forward() : 0);
     return cuda_rc(cudaGetLastError());
 }
@@ -1251,30 +1259,44 @@ int sphfsi_finalize(sphfsi_ctx *c)
     // cell form and with rows: 2-D channels of 33k particles 87 against 71 us,
     // batches of 171k and 577k 248 and 574 against 234 and 485; 3-D tanks of 4k,
     // 11k, 24k and 62k 219, 151, 202 and 393 against 218, 151, 182 and 320.
-    // Smaller 2-D contexts would gain too (a channel of 10k 65 -> 60 us, a dam
-    // break of 14k 90 -> 87), but the form decides the order of the sums, and a
-    // batch of a few thousand particles per instance equals its instances
-    // stepped alone to the last bit: both have to take the same one.
+    // Smaller problems gain little or nothing (2-D channel of 10k 65 -> 60 us, dam
+    // break of 14k 90 -> 87; 3-D as above).
+    // The form decides the order of a particle's sums, and a batch equals its
+    // instances stepped alone to the last bit: an instance of a batch takes the
+    // form that it takes alone.  (Contexts of 262 144 particles and more, whose
+    // launch shape is not that of their instances anyway, go by their total:
+    // 32 channels of 577k in all 574 -> 485 us.)
     F.n = (int)nf;
     c->S.n = (int)ns;
     cell_form(c, F);
-    if (c->max_reach == 1 && nf >= (D == 3 ? 16384 : 32768)) {
+    std::vector<int> form(B, 0);
+    int with_rows = 0;
+    for (int b = 0; b < B; b++) {
+        const int64_t size = small ? c->ih[b].nf : nf;
+        form[b] = c->max_reach == 1 && size >= (D == 3 ? 16384 : 32768) ? 1 : 0;
+        with_rows += form[b];
+    }
+    F.only = -1;
+    int *d_form = nullptr;
+    TRY(dscratch(c, &d_form, B));
+    TRY(upload(c, d_form, form));
+    F.form = d_form;
+    c->two_forms = with_rows > 0 && with_rows < B;
+    if (with_rows) {
         F.list = 1;
         F.lanes = D == 3 ? 4 : 2;
         F.compact = 0;
         F.rows = 0;
     }
     // Is the solid branch longer than rows, momentum and continuity?  From the
-    // first step's K and the measured cost of a sub-step (about 2 us in one
-    // cluster, 5 us in the 2-D window kernel, 8 us in 3-D) against 25 us and 1 ns
-    // per fluid particle in 2-D, 2.5 ns in 3-D.  Dam break of 56k particles and a
-    // body of 6400, 25 sub-steps: step 199 us with the rows first, 185 so.
-    {
-        double K = 0.0;
-        for (int b = 0; b < B; b++) K = std::max(K, first_substeps(c->ih[b]));
-        const double sub = D == 3 ? 8.0 : (max_ns > 2048 ? 5.0 : 2.0);
-        c->fork_first = sub * K > 25.0 + (D == 3 ? 2.5e-3 : 1e-3) * (double)nf;
-    }
+    // first step's K and the measured cost of a sub-step of the window kernel
+    // (about 5 us in 2-D, 8 us in 3-D) against 25 us and 1 ns per fluid particle
+    // in 2-D, 2.5 ns in 3-D.  Dam break of 56k particles and a body of 6400, 25
+    // sub-steps: step 199 us with the rows first, 185 so.  Only for a body beyond
+    // one cluster, which no batch holds: the reinitialisation then sums in the
+    // cells' order.
+    c->fork_first = max_ns > kClusterBody &&
+                    (D == 3 ? 8.0 : 5.0) * first_substeps(c->ih[0]) > 25.0 + (D == 3 ? 2.5e-3 : 1e-3) * (double)nf;
     F.list_lanes = 1;
     F.list_cap = D == 2 ? 64 : 128;
     TRY(dalloc(c, &F.nbl, (size_t)nf * F.list_cap));
@@ -2108,6 +2130,7 @@ int sphfsi_set_tuning(sphfsi_ctx *c, const sphfsi_tuning *t)
     c->F.split_records = t->records == 1 ? 1 : 0;
     c->F.bin_fused = t->records == 2 ? 1 : 0;
     c->F.rows = t->rows;
+    c->two_forms = false;   // one shape for all
     // a held configuration built without rows has none to stream
     if (t->list && !c->F.list && held_on(c->F)) TRY(request_rebuild(c));
     c->F.list = t->list;
@@ -2144,6 +2167,7 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
     TRY(cuda_rc(cudaStreamSynchronize(c->st)));
     sphfsi_tuning cur{}, keep{};
     sphfsi_get_tuning(c, &keep);
+    const bool keep_two = c->two_forms;
     // snapshot of every device allocation of the state, restored before each trial and at the end
     size_t total = 0;
     for (auto &a : c->allocs) total += (a.second + 255) & ~(size_t)255;
@@ -2253,7 +2277,10 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
     int rc2 = copy_all(false);
     if (!rc) rc = rc2;
     if (!rc) rc = sphfsi_set_tuning(c, best);
-    else sphfsi_set_tuning(c, &keep);
+    else {
+        sphfsi_set_tuning(c, &keep);
+        c->two_forms = keep_two;
+    }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(snap);

@@ -221,6 +221,10 @@ struct Fluid {
     // restored nbc (launch_row_parts)
     int *part[2];
     int *part_n;
+    // a context whose instances differ in form (sphfsi_finalize): the pair
+    // kernels run once per form, over the instances of it
+    const int *form;      // per instance: 1 rows, 0 cells
+    int only;             // the form this launch takes; -1: every instance
     float4 *B4;           // boundary part of a target's density rate: coefficient on v^{n+1}, constant
 };
 
@@ -248,6 +252,8 @@ struct Walls {
 
 // Elastic bodies (device locality order within each instance) + their
 // records in the fluid grid.
+constexpr int kClusterBody = 2048;   // largest body of one thread-block cluster (16 CTAs of 128 particles)
+
 struct Solid {
     int n;
     int nnz;
@@ -351,6 +357,9 @@ __device__ __forceinline__ bool rebuild_step(const Batch &bt, const Fluid &f)
     if (f.held_n == 0) return f.held[2] != 0;   // automatic: the last step's finish kernel decided
     return bt.ctl[0].step % f.held_n == 0;
 }
+
+// does a launch of the pair kernels take instance b?
+__device__ __forceinline__ bool takes(const Fluid &f, int b) { return f.only < 0 || f.form[b] == f.only; }
 
 // the pair configuration is held over several steps (fixed or automatic cadence)
 __device__ __host__ __forceinline__ bool held_on(const Fluid &f) { return f.held_n != 1; }

@@ -16,7 +16,7 @@ template <int D, int L, bool CP, int FORM>
 __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int i,
                                                  bool act_, int lane, uint32_t *list, int stride, const TileSrc *ts)
 {
-    const bool act = act_;
+    const bool act = act_ && (f.only < 0 || takes(f, f.inst[i]));
     const int b = act ? f.inst[i] : 0;
     const Inst &In = bt.I[b];
     const Grid &g = In.g;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kMaxBlock, D == 2 && FORM != 1 ? 5 : (D == 3 &
     const int stride = blockDim.x, lane = (int)threadIdx.x % L;
     constexpr int SETS = FORM == 3 ? kFluidWall : kAllSets;
     // is this a reinitialisation step of target i's instance?
-    auto due = [&](int i) { return i < f.n && bt.ctl[f.inst[i]].reinit; };
+    auto due = [&](int i) { return i < f.n && bt.ctl[f.inst[i]].reinit && takes(f, f.inst[i]); };
     if constexpr (!TILE) {
         const int nn = FORM == 3 ? part_blocks(f.n, kPartNear, blockDim.x) : 0;
         if ((int)blockIdx.x < nn) {

@@ -21,7 +21,8 @@ template <int D, int L, bool CP, int FORM, int SETS>
 __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int i,
                                                  bool act_, int lane, uint32_t *list, int stride, const TileSrc *ts)
 {
-    const bool act = act_ && (SETS != kFluidOnly || !(f.nbc[i] & (kListSolid | kListWalls | kListOver)));
+    const bool act = act_ && (SETS != kFluidOnly || !(f.nbc[i] & (kListSolid | kListWalls | kListOver))) &&
+                     (f.only < 0 || takes(f, f.inst[i]));
     const int b = act ? f.inst[i] : 0;
     const Inst &In = bt.I[b];
     const Grid &g = In.g;
@@ -339,6 +340,10 @@ __global__ void __launch_bounds__(32 * kRowWarps, D == 3 ? 5 : 8) k_pairlist_cel
     const int a0 = f.cstart[cell], a1 = f.cstart[cell + 1];
     if (a0 >= a1) return;
     RowWarp<D> &sw = s_warp[threadIdx.x >> 5];
+    if (!takes(f, f.inst[a0])) {
+        if (a0 == 0 && lane == 0) f.nbc[0] = kListBuilt;   // (the other instances' rows are)
+        return;
+    }
     const Inst &In = bt.I[f.inst[a0]];
     const Grid &g = In.g;
     const float rc2 = In.P.rc2F, reach2 = rc2 * 1.0001f;   // the box test's rounding stays within the margin

@@ -371,6 +371,7 @@ constexpr int kCThreads = 512;
 constexpr int kLanes = 4;
 constexpr int kPPC = kCThreads / kLanes;
 constexpr int kClusterMax = 16;
+static_assert(kClusterMax * kPPC == kClusterBody && kClusterMax * kSolidCta == kClusterBody, "one cluster's body");
 
 __device__ __forceinline__ unsigned cluster_rank()
 {
