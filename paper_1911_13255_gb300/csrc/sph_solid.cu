@@ -401,6 +401,53 @@ __device__ __forceinline__ float group_sum(float v)
     return v;
 }
 
+// 3-D: the eight strands (below), two per lane
+__device__ __forceinline__ float strand_sum(float a, float b)
+{
+    float v = __fadd_rn(a, b);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
+}
+
+// Arithmetic that the 3-D cluster kernel and the windowed kernel share.  A body
+// of up to one cluster's size takes the one in a batch and the other alone, and
+// has to come out the same to the last bit: a particle's sums run over eight
+// strands (every eighth entry of its list; eight lanes in the windowed kernel,
+// two strands in each of four lanes in the cluster kernel), added in the order
+// strand + 4, + 2, + 1, and every operation that the compiler could contract in
+// two ways is written out.
+__device__ __forceinline__ void pair_rate3(float *M, const float *dv, const float4 &e)
+{
+    const float ge[3] = {e.x, e.y, e.z};
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) M[3 * i + j] = __fmaf_rn(dv[i], ge[j], M[3 * i + j]);
+}
+__device__ __forceinline__ float pair_force3(float sum, const float4 &qa, const float4 &qb, const float4 &e)
+{
+    const float t = __fmaf_rn(qa.z + qb.z, e.z, __fmaf_rn(qa.y + qb.y, e.y, __fmul_rn(qa.x + qb.x, e.x)));
+    return __fadd_rn(sum, t);
+}
+// sum += d; rest: what the FP32 sum has rounded off so far this step, carried
+// into the next addition, so that a step rounds its state once instead of at
+// every sub-step
+__device__ __forceinline__ void add_rest(float &sum, float &rest, float d)
+{
+    const float y = __fadd_rn(d, rest), t = __fadd_rn(sum, y);
+    rest = __fsub_rn(y, __fsub_rn(t, sum));
+    sum = t;
+}
+__device__ __forceinline__ float solid_accel(float sum, float inv_rho, float fF, float inv_m, float g)
+{
+    return __fadd_rn(__fmaf_rn(sum, inv_rho, __fmul_rn(fF, inv_m)), g);
+}
+__device__ __forceinline__ float square3(float x, float y, float z)
+{
+    return __fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x)));
+}
+
 // K sub-steps of one instance's body (slots [s0, s0 + ns)) by one cluster
 template <int D>
 __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, Ctl *ctl, int s0, int ns, float4 *sQ,
@@ -417,6 +464,7 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
     const float inv_rhoS = 1.0f / P.rhoS, inv_mS = 1.0f / P.mS;
 
     float H[9], B[9], fF[3] = {0.f, 0.f, 0.f};
+    float Hr[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, vr[3] = {0.f, 0.f, 0.f};   // 3-D: rests of H and v (add_rest)
     double x = 0, y = 0, z = 0, xs = 0, ys = 0, zs = 0, as[3] = {0, 0, 0};
     bool cons = true;
     float vmax = 0.0f, amax = 0.0f;
@@ -444,7 +492,7 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
     // in flight together.
     constexpr int kU = 4;
     auto rate = [&](float4 va, float *Hd) {
-        float M[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        float M[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, M2[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // 3-D: the lane's two strands
         for (int base = q0 + lane; base < q1; base += kLanes * kU) {
             float4 e[kU], vb[kU];
 #pragma unroll
@@ -461,18 +509,28 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
 #pragma unroll
             for (int u = 0; u < kU; u++) {
                 float dv[3] = {vb[u].x - va.x, vb[u].y - va.y, vb[u].z - va.z};
-                float ge[3] = {e[u].x, e[u].y, e[u].z};
-                for (int i = 0; i < D; i++)
-                    for (int j = 0; j < D; j++) M[i * D + j] += dv[i] * ge[j];
+                if (D == 3) {
+                    pair_rate3(u & 1 ? M2 : M, dv, e[u]);
+                } else {
+                    float ge[3] = {e[u].x, e[u].y, e[u].z};
+                    for (int i = 0; i < D; i++)
+                        for (int j = 0; j < D; j++) M[i * D + j] += dv[i] * ge[j];
+                }
             }
         }
-        for (int i = 0; i < D * D; i++) M[i] = group_sum(M[i]);
+        for (int i = 0; i < D * D; i++) M[i] = D == 3 ? strand_sum(M[i], M2[i]) : group_sum(M[i]);
         for (int i = 0; i < D; i++)
             for (int j = 0; j < D; j++) {
                 float v = 0.0f;
-                for (int k = 0; k < D; k++) v += M[i * D + k] * B[k * D + j];
+                for (int k = 0; k < D; k++) v = __fmaf_rn(M[i * D + k], B[k * D + j], v);
                 Hd[i * D + j] = v;
             }
+    };
+    auto drift_H = [&](const float *Hd) {
+        for (int i = 0; i < D * D; i++) {
+            if (D == 3) add_rest(H[i], Hr[i], __fmul_rn(hdts, Hd[i]));
+            else H[i] = H[i] + hdts * Hd[i];
+        }
     };
     auto put_Q = [&]() {
         float Q[9];
@@ -494,11 +552,11 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
         float Hd[9];
         rate(va, Hd);
         if (own && lane == 0) {
-            for (int i = 0; i < D * D; i++) H[i] = H[i] + hdts * Hd[i];
+            drift_H(Hd);
             if (!cons) {
-                x = x + hdtsd * (double)va.x;
-                y = y + hdtsd * (double)va.y;
-                if (D == 3) z = z + hdtsd * (double)va.z;
+                x = __fma_rn(hdtsd, (double)va.x, x);
+                y = __fma_rn(hdtsd, (double)va.y, y);
+                if (D == 3) z = __fma_rn(hdtsd, (double)va.z, z);
             }
             put_Q();
         }
@@ -519,7 +577,7 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
                     }
                 }
             }
-            float acc[3] = {0.f, 0.f, 0.f};
+            float acc[3] = {0.f, 0.f, 0.f}, acc2[3] = {0.f, 0.f, 0.f};
             for (int base = q0 + lane; base < q1; base += kLanes * kU) {
                 float4 e[kU];
 #pragma unroll
@@ -549,29 +607,31 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
                         unsigned rb = (unsigned)(b / kPPC);
                         int lb = b % kPPC;
                         for (int r = 0; r < 3; r++) {
-                            float4 qv = *dsmem(&sQ[3 * lb + r], rb);
-                            acc[r] += (Qa[3 * r] + qv.x) * e[u].x + (Qa[3 * r + 1] + qv.y) * e[u].y +
-                                      (Qa[3 * r + 2] + qv.z) * e[u].z;
+                            const float4 qv = *dsmem(&sQ[3 * lb + r], rb);
+                            const float4 qa = make_float4(Qa[3 * r], Qa[3 * r + 1], Qa[3 * r + 2], 0.0f);
+                            float &f = u & 1 ? acc2[r] : acc[r];
+                            f = pair_force3(f, qa, qv, e[u]);
                         }
                     }
                 }
             }
-            for (int k = 0; k < D; k++) acc[k] = group_sum(acc[k]);
+            for (int k = 0; k < D; k++) acc[k] = D == 3 ? strand_sum(acc[k], acc2[k]) : group_sum(acc[k]);
             if (own && lane == 0 && !cons) {
                 float4 v = sV[g];
-                float av[3];
-                for (int k = 0; k < D; k++) av[k] = acc[k] * inv_rhoS + fF[k] * inv_mS + P.g[k];
-                v.x += dts * av[0];
-                v.y += dts * av[1];
-                if (D == 3) v.z += dts * av[2];
-                sV[g] = v;
-                float a2 = 0.0f;
-                for (int k = 0; k < D; k++) {
-                    as[k] += dtsd * (double)av[k];
-                    a2 += av[k] * av[k];
+                float av[3] = {0.f, 0.f, 0.f};
+                for (int k = 0; k < D; k++) av[k] = solid_accel(acc[k], inv_rhoS, fF[k], inv_mS, P.g[k]);
+                if (D == 3) {
+                    add_rest(v.x, vr[0], __fmul_rn(dts, av[0]));
+                    add_rest(v.y, vr[1], __fmul_rn(dts, av[1]));
+                    add_rest(v.z, vr[2], __fmul_rn(dts, av[2]));
+                } else {
+                    v.x += dts * av[0];
+                    v.y += dts * av[1];
                 }
-                amax = max_keep_nan(amax, a2);
-                vmax = max_keep_nan(vmax, v.x * v.x + v.y * v.y + v.z * v.z);
+                sV[g] = v;
+                for (int k = 0; k < D; k++) as[k] = __fma_rn(dtsd, (double)av[k], as[k]);
+                amax = max_keep_nan(amax, square3(av[0], av[1], av[2]));
+                vmax = max_keep_nan(vmax, square3(v.x, v.y, v.z));
             }
         }
         cluster_sync();
@@ -582,20 +642,14 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
             float Hd[9];
             rate(va, Hd);
             if (own && lane == 0) {
-                for (int i = 0; i < D * D; i++) {
-                    H[i] = H[i] + hdts * Hd[i];
-                    if (more) H[i] = H[i] + hdts * Hd[i];
-                }
-                if (!cons) {
-                    x = x + hdtsd * (double)va.x;
-                    y = y + hdtsd * (double)va.y;
-                    if (D == 3) z = z + hdtsd * (double)va.z;
-                    if (more) {
-                        x = x + hdtsd * (double)va.x;
-                        y = y + hdtsd * (double)va.y;
-                        if (D == 3) z = z + hdtsd * (double)va.z;
+                drift_H(Hd);
+                if (more) drift_H(Hd);
+                if (!cons)
+                    for (int r = 0; r < (more ? 2 : 1); r++) {
+                        x = __fma_rn(hdtsd, (double)va.x, x);
+                        y = __fma_rn(hdtsd, (double)va.y, y);
+                        if (D == 3) z = __fma_rn(hdtsd, (double)va.z, z);
                     }
-                }
                 if (more) put_Q();
             }
         }
@@ -1654,10 +1708,14 @@ __global__ void __launch_bounds__(kWinThreads, 1) k_solid_window(Batch bt, Solid
             [&](const float4 &e, int ib) {
                 const float4 vb = sV[ib];
                 const float dv[3] = {vb.x - va.x, vb.y - va.y, vb.z - va.z}, ge[3] = {e.x, e.y, e.z};
+                if constexpr (D == 3) {
+                    pair_rate3(M, dv, e);
+                } else {
 #pragma unroll
-                for (int i = 0; i < D; i++)
+                    for (int i = 0; i < D; i++)
 #pragma unroll
-                    for (int j = 0; j < D; j++) M[i * D + j] += dv[i] * ge[j];
+                        for (int j = 0; j < D; j++) M[i * D + j] += dv[i] * ge[j];
+                }
             },
             [&](bool act, int p) {
 #pragma unroll
@@ -1684,10 +1742,7 @@ __global__ void __launch_bounds__(kWinThreads, 1) k_solid_window(Batch bt, Solid
                     f[1] += (qa[0].z + qb.z) * e.x + (qa[0].w + qb.w) * e.y;
                 } else {
 #pragma unroll
-                    for (int r = 0; r < QR; r++) {
-                        const float4 qb = sQ[r * s.win_slots + ib];
-                        f[r] += (qa[r].x + qb.x) * e.x + (qa[r].y + qb.y) * e.y + (qa[r].z + qb.z) * e.z;
-                    }
+                    for (int r = 0; r < QR; r++) f[r] = pair_force3(f[r], qa[r], sQ[r * s.win_slots + ib], e);
                 }
             },
             [&](bool act, int p) {
@@ -1702,20 +1757,13 @@ __global__ void __launch_bounds__(kWinThreads, 1) k_solid_window(Batch bt, Solid
     // state of particle t
     const bool own = t < n;
     const int a = a0 + (own ? t : 0), slot = a - lo;
-    // (Hr, vr: what the FP32 sums H and v have rounded off so far this step,
-    // carried into the next addition, so that a step rounds its state once
-    // instead of at every sub-step)
+    // (Hr, vr: the rests of H and v, add_rest)
     float H[DD], B[DD], fF[3] = {0.f, 0.f, 0.f}, vmax = 0.0f, amax = 0.0f;
     float Hr[DD], vr[3] = {0.f, 0.f, 0.f};
     double x = 0, y = 0, z = 0, xs = 0, ys = 0, zs = 0, as[3] = {0, 0, 0};
     bool cons = true;
 #pragma unroll
     for (int i = 0; i < DD; i++) Hr[i] = 0.0f;
-    auto add = [](float &sum, float &rest, float d) {
-        const float y = __fadd_rn(d, rest), t = __fadd_rn(sum, y);
-        rest = __fsub_rn(y, __fsub_rn(t, sum));
-        sum = t;
-    };
     if (own) {
 #pragma unroll
         for (int i = 0; i < DD; i++) {
@@ -1743,17 +1791,18 @@ __global__ void __launch_bounds__(kWinThreads, 1) k_solid_window(Batch bt, Solid
                 for (int j = 0; j < D; j++) {
                     float hd = 0.0f;
 #pragma unroll
-                    for (int k = 0; k < D; k++) hd += M[i * D + k] * B[k * D + j];
-                    if (second) add(H[i * D + j], Hr[i * D + j], hdts * hd);
-                    if (first) add(H[i * D + j], Hr[i * D + j], hdts * hd);
+                    for (int k = 0; k < D; k++) hd = __fmaf_rn(M[i * D + k], B[k * D + j], hd);
+                    const float dh = __fmul_rn(hdts, hd);
+                    if (second) add_rest(H[i * D + j], Hr[i * D + j], dh);
+                    if (first) add_rest(H[i * D + j], Hr[i * D + j], dh);
                 }
             if (!cons) {
                 const float4 v = sV[slot];
                 const int reps = (second ? 1 : 0) + (first ? 1 : 0);
                 for (int r = 0; r < reps; r++) {
-                    x = x + hdtsd * (double)v.x;
-                    y = y + hdtsd * (double)v.y;
-                    if (D == 3) z = z + hdtsd * (double)v.z;
+                    x = __fma_rn(hdtsd, (double)v.x, x);
+                    y = __fma_rn(hdtsd, (double)v.y, y);
+                    if (D == 3) z = __fma_rn(hdtsd, (double)v.z, z);
                 }
             }
             if (first) {
@@ -1783,21 +1832,20 @@ __global__ void __launch_bounds__(kWinThreads, 1) k_solid_window(Batch bt, Solid
         load_Q();
         force_sums();
         if (own && !cons) {
-            float av[3] = {0.f, 0.f, 0.f}, a2 = 0.0f;
+            float av[3] = {0.f, 0.f, 0.f};
             float4 v = sV[slot];
 #pragma unroll
             for (int k = 0; k < D; k++) {
-                av[k] = sM[t * DD + k] * inv_rhoS + fF[k] * inv_mS + P.g[k];
-                as[k] += dtsd * (double)av[k];
-                a2 += av[k] * av[k];
+                av[k] = solid_accel(sM[t * DD + k], inv_rhoS, fF[k], inv_mS, P.g[k]);
+                as[k] = __fma_rn(dtsd, (double)av[k], as[k]);
             }
-            add(v.x, vr[0], dts * av[0]);
-            add(v.y, vr[1], dts * av[1]);
-            if (D == 3) add(v.z, vr[2], dts * av[2]);
+            add_rest(v.x, vr[0], __fmul_rn(dts, av[0]));
+            add_rest(v.y, vr[1], __fmul_rn(dts, av[1]));
+            if (D == 3) add_rest(v.z, vr[2], __fmul_rn(dts, av[2]));
             sV[slot] = v;
             __stcg(&s.v4[a], v);
-            amax = max_keep_nan(amax, a2);
-            vmax = max_keep_nan(vmax, v.x * v.x + v.y * v.y + v.z * v.z);
+            amax = max_keep_nan(amax, square3(av[0], av[1], av[2]));
+            vmax = max_keep_nan(vmax, square3(v.x, v.y, v.z));
         }
         publish();
         // (C) deformation rate at v^{k+1}, second half drift; next first half and stress
