@@ -1303,7 +1303,7 @@ int sphfsi_finalize(sphfsi_ctx *c)
     TRY(dalloc(c, &F.nbc, nf));
     for (int p = 0; p < 2; p++) TRY(dscratch(c, &F.part[p], nf));
     TRY(dscratch(c, &F.part_n, 2));
-    TRY(dscratch(c, &F.B4, nf));
+    TRY(dscratch(c, &F.bnd, nf));
     // held pair configuration: off (rebuilt every step); the first step builds it
     F.held_n = 1;
     TRY(dalloc(c, &F.held, 3));

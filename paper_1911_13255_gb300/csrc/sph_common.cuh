@@ -225,7 +225,7 @@ struct Fluid {
     // kernels run once per form, over the instances of it
     const int *form;      // per instance: 1 rows, 0 cells
     int only;             // the form this launch takes; -1: every instance
-    float4 *B4;           // boundary part of a target's density rate: coefficient on v^{n+1}, constant
+    float *bnd;           // boundary part of a target's density rate / (2 rho) at v^{n+1}
 };
 
 // nbc flags: solid particles in one of the target's neighbour cells (the pair

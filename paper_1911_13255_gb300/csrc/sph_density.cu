@@ -50,10 +50,7 @@ __device__ __forceinline__ void density_one(const Batch &bt, const Fluid &f, con
     rate = group_sum<L>(rate);
     if (!act || lane != 0) return;
     // walls and solid: the momentum loop's sums (fs_pair_force)
-    if (FORM != 3 || (f.nbc[i] & (kListSolid | kListWalls | kListOver))) {
-        const float4 Bi = f.B4[i];
-        rate += Bi.x * Wi.x + Bi.y * Wi.y + (D == 3 ? Bi.z * Wi.z : 0.0f) + Bi.w;
-    }
+    if (FORM != 3 || (f.nbc[i] & (kListSolid | kListWalls | kListOver))) rate += f.bnd[i];
     const float vi[3] = {Wi.x, Wi.y, Wi.z};
     const float rhoi = P.rho0 + Wi.w;
     float rhodot = 2.0f * rhoi * rate;

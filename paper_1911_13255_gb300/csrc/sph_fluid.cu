@@ -14,8 +14,8 @@ namespace sph {
 // ---------------------------------------------------------------------------
 // a4: equation of state + momentum + kick
 // ---------------------------------------------------------------------------
-// Also sums the boundary part of the continuity equation of target i (its
-// coefficient on v^{n+1} and its constant, fs_pair_force) into B4.
+// Also leaves the boundary part of target i's continuity equation at v^{n+1}
+// (fs_pair_force) in bnd.
 // SETS: what the loop visits; kFluidOnly skips the listed targets (row form).
 template <int D, int L, bool CP, int FORM, int SETS>
 __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, const Walls &w, const Solid &s, int i,
@@ -108,7 +108,11 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
             f.dvdt[(size_t)i * D + k] = a[k];
         }
         f.W4[i] = make_float4(vn[0], vn[1], vn[2], Vi.w);
-        if (SETS != kFluidOnly) f.B4[i] = make_float4(bnd[0], bnd[1], bnd[2], bnd[3]);
+        if (SETS != kFluidOnly) {
+            float r = bnd[3];
+            for (int k = 0; k < D; k++) r += bnd[k] * (vn[k] - vi[k]);
+            f.bnd[i] = r;
+        }
         cnt.vmax = sqrtf(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
         // a position that is no number is in nobody's support where rows or
         // compacted lists are tested with "<": the finish kernel hears of it here

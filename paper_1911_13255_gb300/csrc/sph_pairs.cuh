@@ -801,10 +801,12 @@ __device__ __forceinline__ void cell_xyz(int gkey, const Inst &In, int &cx, int 
 // rho^d), only its normal part enters),
 //   V_a (-dW) [(v~_a - v).d / r + (p^d - p_i) / ((rho_i + rho^d) c0)],
 // times 2 rho_i.  It is taken at the velocity v^{n+1} that the forces are yet
-// to give, but it is affine in v, so the momentum loop sums its coefficient
-// (rate[0..2], to be multiplied by v) and its constant (rate[3]) while it has
-// the pair's geometry and ghost state, and the continuity loop visits no
-// boundary particle (continuity, 2-D flag channel 20.6 -> 12.2 us, dam break
+// to give, but it is affine in v, so the momentum loop sums its value at v_i
+// (rate[3]) and its coefficient on v^{n+1} - v_i (rate[0..2]) while it has the
+// pair's geometry and ghost state, and the continuity loop visits no boundary
+// particle.  About v_i, so that what body and fluid have in common cancels in
+// every pair: sums about v = 0 leave the rounding of that velocity, and a body
+// that moves along with its fluid gets a rate (continuity, 2-D flag channel 20.6 -> 12.2 us, dam break
 // 22.4 -> 13.3 us, batch of 32 channels 243 -> 176 us; 3-D duct 1.70 -> 1.02 ms).
 template <int D>
 __device__ __forceinline__ void fs_pair_force(const float d[3], float r2, const float vi[3], float rhoi, float pi,
@@ -837,12 +839,12 @@ __device__ __forceinline__ void fs_pair_force(const float d[3], float r2, const 
         const float w = Va * dW, wr = w * invr;
         rate[0] += wr * d[0];
         rate[1] += wr * d[1];
-        float vd = vb.x * d[0] + vb.y * d[1];
+        float vd = (vi[0] - vb.x) * d[0] + (vi[1] - vb.y) * d[1];
         if (D == 3) {
             rate[2] += wr * d[2];
-            vd += vb.z * d[2];
+            vd += (vi[2] - vb.z) * d[2];
         }
-        rate[3] -= wr * vd + w * dpg / (rsum * P.c0);
+        rate[3] += wr * vd - w * dpg / (rsum * P.c0);
     }
 }
 
