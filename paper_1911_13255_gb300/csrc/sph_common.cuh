@@ -464,7 +464,7 @@ __device__ __forceinline__ float eos_p(float drho, const Phys &P)
 // inverse (ghost density), rho = rho0 (1 + p / p_coef)^(1/7)
 __device__ __forceinline__ float eos_rho(float p, const Phys &P)
 {
-    return P.rho0 * expf(log1pf(p * P.inv_p_coef) * (1.0f / 7.0f));
+    return __fmul_rn(P.rho0, expf(__fmul_rn(log1pf(__fmul_rn(p, P.inv_p_coef)), 1.0f / 7.0f)));
 }
 
 // Wendland C2 derivative dW/dr at h_F (Section 4); caller guarantees q < 2

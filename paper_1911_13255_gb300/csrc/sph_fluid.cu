@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) k_solid_fluid_force(Batch bt, Fl
             const float4 Pj = f.P4[j];
             // the fluid side sees this pair with the opposite cell offset
             float d[3] = {(Pj.x - A.x) - ox, (Pj.y - A.y) - oy, D == 3 ? (Pj.z - A.z) - oz : 0.0f};
-            float r2 = d[0] * d[0] + d[1] * d[1] + (D == 3 ? d[2] * d[2] : 0.0f);
+            const float r2 = square_norm<D>(d);
             if (r2 >= P.rc2F) return;
             nsf++;
             const float4 Vj = f.V4[j];

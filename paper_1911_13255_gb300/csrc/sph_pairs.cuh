@@ -188,13 +188,21 @@ __device__ __forceinline__ uint4 transpose4(uint4 e, int lane, unsigned group)
     return e;
 }
 
+// |d|^2, one sequence of operations wherever a pair's distance is taken
+template <int D>
+__device__ __forceinline__ float square_norm(const float d[3])
+{
+    const float s = __fmaf_rn(d[0], d[0], __fmul_rn(d[1], d[1]));
+    return D == 3 ? __fmaf_rn(d[2], d[2], s) : s;
+}
+
 template <int D>
 __device__ __forceinline__ float rel_d(const float4 &Pi, const float4 &Pj, float ox, float oy, float oz, float d[3])
 {
     d[0] = (Pi.x - Pj.x) + ox;
     d[1] = (Pi.y - Pj.y) + oy;
     d[2] = D == 3 ? (Pi.z - Pj.z) + oz : 0.0f;
-    return d[0] * d[0] + d[1] * d[1] + (D == 3 ? d[2] * d[2] : 0.0f);
+    return square_norm<D>(d);
 }
 
 // the same for row entry e: (P_i - P_j) + o with o = step * edge, which one fused
@@ -212,7 +220,7 @@ __device__ __forceinline__ float rel_row(const float4 &Pi, const float4 &Pj, uin
     d[0] = __fmaf_rn(row_step(e, 0), c.x, Pi.x - Pj.x);
     d[1] = __fmaf_rn(row_step(e, 1), c.y, Pi.y - Pj.y);
     d[2] = D == 3 ? __fmaf_rn(row_step(e, 2), c.z, Pi.z - Pj.z) : 0.0f;
-    return d[0] * d[0] + d[1] * d[1] + (D == 3 ? d[2] * d[2] : 0.0f);
+    return square_norm<D>(d);
 }
 
 // ---------------------------------------------------------------------------
@@ -793,8 +801,10 @@ __device__ __forceinline__ void cell_xyz(int gkey, const Inst &In, int &cx, int 
 // its volume V_i, i.e. V_a [-2 p_bar dW/r d + 4 eta (v_i - v~_a) dW / (r + 0.01 h_F)]
 // (Eqs. fs-force-mr-sp, fs-force-mr-sv with v_i - v^d_a = 2 (v_i - v~_a),
 // reading R6: p^d = p_i + rho_i max(0, -(g - a~).n) max(0, r_ia.n), rho^d from
-// the inverse EoS).  Identical arithmetic on the fluid and the solid side,
-// so each pair's term is bitwise antisymmetric.
+// the inverse EoS).  The fluid and the solid side call it with the same
+// numbers, and every operation that the compiler could contract in two ways is
+// written out (also in square_norm, whose r^2 both pass in): each pair's
+// term is bitwise antisymmetric whatever else the loops around it hold.
 //
 // With rate, also the pair's part of the continuity equation (reading R7: the
 // Riemann interface velocity between (v, p_i, rho_i) and the ghost (v^d, p^d,
@@ -819,23 +829,23 @@ __device__ __forceinline__ void fs_pair_force(const float d[3], float r2, const 
     float r = sqrtf(r2);
     float invr = r2 > 0.0f ? 1.0f / r : 0.0f;
     float dW = dW_F(r, P);
-    float gn = (P.g[0] - ab.x) * n.x + (P.g[1] - ab.y) * n.y;
-    float dn = d[0] * n.x + d[1] * n.y;
+    float gn = __fmaf_rn(P.g[0] - ab.x, n.x, __fmul_rn(P.g[1] - ab.y, n.y));
+    float dn = __fmaf_rn(d[0], n.x, __fmul_rn(d[1], n.y));
     if (D == 3) {
-        gn += (P.g[2] - ab.z) * n.z;
-        dn += d[2] * n.z;
+        gn = __fmaf_rn(P.g[2] - ab.z, n.z, gn);
+        dn = __fmaf_rn(d[2], n.z, dn);
     }
-    float dpg = rhoi * fmaxf(0.0f, -gn) * fmaxf(0.0f, dn);   // p^d - p_i
-    float pd = pi + dpg;
-    float rhod = eos_rho(pd, P);
-    float rsum = rhoi + rhod;
-    float pbar = (pi * rhod + pd * rhoi) / rsum;
-    float sp = -2.0f * pbar * dW * invr;
-    float sv = 4.0f * P.eta * dW / (r + P.hreg);
-    out[0] = Va * (sp * d[0] + sv * (vi[0] - vb.x));
-    out[1] = Va * (sp * d[1] + sv * (vi[1] - vb.y));
-    out[2] = D == 3 ? Va * (sp * d[2] + sv * (vi[2] - vb.z)) : 0.0f;
+    const float push = __fmul_rn(rhoi, fmaxf(0.0f, -gn)), lift = fmaxf(0.0f, dn);
+    const float pd = __fmaf_rn(push, lift, pi);
+    const float rhod = eos_rho(pd, P), rsum = __fadd_rn(rhoi, rhod);
+    const float pbar = __fdiv_rn(__fmaf_rn(pi, rhod, __fmul_rn(pd, rhoi)), rsum);
+    const float sp = __fmul_rn(__fmul_rn(__fmul_rn(-2.0f, pbar), dW), invr);
+    const float sv = __fdiv_rn(__fmul_rn(__fmul_rn(4.0f, P.eta), dW), __fadd_rn(r, P.hreg));
+    out[0] = __fmul_rn(Va, __fmaf_rn(sp, d[0], __fmul_rn(sv, vi[0] - vb.x)));
+    out[1] = __fmul_rn(Va, __fmaf_rn(sp, d[1], __fmul_rn(sv, vi[1] - vb.y)));
+    out[2] = D == 3 ? __fmul_rn(Va, __fmaf_rn(sp, d[2], __fmul_rn(sv, vi[2] - vb.z))) : 0.0f;
     if (rate) {
+        const float dpg = __fmul_rn(push, lift);   // p^d - p_i
         const float w = Va * dW, wr = w * invr;
         rate[0] += wr * d[0];
         rate[1] += wr * d[1];
