@@ -114,17 +114,24 @@ int launch_density(const Batch &bt, const Fluid &f, const Walls &w, const Solid 
 // given that way.  Per-particle sums are finished in FP64.
 //
 // What bounds the loop is FP32 issue, so the pairs are kept short:
-//  - hi of a position is rounded to a fixed quantum, 2^-21 of a power of two
-//    above the cell edge, and so is hi of the edge: differences of hi parts are
-//    then exact, one addition instead of a TwoSum (Knuth) each;
+//  - a position's FP32 number is cut at a fixed quantum, 2^-21 of a power of
+//    two above the cell edge, and so is the edge's: the differences of the upper
+//    and of the lower parts are then exact, one addition each instead of a TwoSum
+//    (Knuth), and so is their sum with its remainder (Dekker), to which the
+//    differences of the records' remainders are added;
 //  - the shape (1 - s)^4 (1 + 4 s), s = r / 2h, takes r as FP32 root s plus
 //    Newton remainder; the remainder rides on the lo parts of 1 - s and 1 + 4 s,
-//    whose hi parts are exact or one FMA from it (Dekker), and no intermediate
-//    sum is renormalised: a product's lo part is good to 2^-48 without.
-// About 96 instructions a pair instead of 190 with general double-float
-// additions and products (3-D duct, 3.0M particles, 714 -> 459 us per step with a
-// reinitialisation every third; 375k 107 -> 75 us); error of a pair against FP64
-// 2e-13 to 5e-13 rms, 2e-11 at most, of a shape between 0 and 1.
+//    whose hi parts are exact or one FMA from it (Dekker), and no product is
+//    renormalised.
+// Measured (general double-float additions and products -> cut parts with one
+// FP32 number for lower part and remainder -> this; per step with a
+// reinitialisation every third): 3-D duct, 3.0M particles 714 -> 448 -> 494 us,
+// 375k 107 -> 75 -> 81, tank of 62k 33 -> 23 -> 23.
+// Error of a shape (between 0 and 1) against 64 bits, restated on the CPU over
+// 400 000 3-D pairs: 8e-15 rms, 1.6e-13 at most; general double-float
+// arithmetic, every operation renormalised, 2e-15 and 2e-14; with the lower parts
+// and the remainders in one FP32 number 2.4e-13 and 3e-12.  The density it ends in
+// is stored as an FP32 deviation, 6e-8 of it.
 // ---------------------------------------------------------------------------
 struct ff {
     float hi, lo;
@@ -143,17 +150,17 @@ __device__ __forceinline__ ff ff_two_sum(float a, float b)
 template <int D>
 struct WendlandPairs {
     float big;                  // x + big - big rounds x to the quantum
-    float edge_hi[3], edge_lo[3], inv_edge[3];
+    float edge_hi[3], edge_mid[3], edge_lo[3], inv_edge[3];
     ff scale;                   // 1 / (4 h^2)
-    float hi[3], lo[3];         // the target
+    float hi[3], mid[3], lo[3]; // the target: upper and lower part of its FP32 position, remainder
 
-    __device__ __forceinline__ void split(const float4 &X, const float4 &R, float h[3], float l[3]) const
+    __device__ __forceinline__ void split(const float4 &X, float h[3], float m[3]) const
     {
-        const float x[3] = {X.x, X.y, X.z}, r[3] = {R.x, R.y, R.z};
+        const float x[3] = {X.x, X.y, X.z};
 #pragma unroll
         for (int k = 0; k < D; k++) {
             h[k] = __fsub_rn(__fadd_rn(x[k], big), big);
-            l[k] = __fadd_rn(__fsub_rn(x[k], h[k]), r[k]);
+            m[k] = __fsub_rn(x[k], h[k]);
         }
     }
     __device__ __forceinline__ WendlandPairs(const Grid &g, const Phys &P, const float4 &Pi, const float4 &Li)
@@ -164,31 +171,36 @@ struct WendlandPairs {
         big = 6.0f * __int_as_float(((__float_as_int(most) >> 23) + 1) << 23);
         for (int k = 0; k < D; k++) {
             edge_hi[k] = __fsub_rn(__fadd_rn(g.csf[k], big), big);
-            edge_lo[k] = __fadd_rn(__fsub_rn(g.csf[k], edge_hi[k]), g.cslo[k]);
+            edge_mid[k] = __fsub_rn(g.csf[k], edge_hi[k]);
+            edge_lo[k] = g.cslo[k];
             inv_edge[k] = 1.0f / g.csf[k];
         }
         const float ih = 0.5f * P.ihF_hi, il = 0.5f * P.ihF_lo;
         scale.hi = __fmul_rn(ih, ih);
         scale.lo = __fmaf_rn(2.0f * ih, il, __fmaf_rn(ih, ih, -scale.hi));
-        split(Pi, Li, hi, lo);
+        split(Pi, hi, mid);
+        lo[0] = Li.x, lo[1] = Li.y, lo[2] = Li.z;
     }
     // adds the shape of the pair with the particle at X (+ remainder R) in the
     // cell of offset o to sum; beyond the support (the screen lets pairs up to
     // 1.0001 (2h)^2 pass) it is below 1e-16
     __device__ __forceinline__ void add(ff &sum, const float4 &X, const float4 &R, float ox, float oy, float oz) const
     {
-        const float o[3] = {ox, oy, oz};
-        float h[3], l[3], d[3], dl[3], p[3], e = 0.0f, c = 0.0f;
-        split(X, R, h, l);
+        const float o[3] = {ox, oy, oz}, l[3] = {R.x, R.y, R.z};
+        float h[3], m[3], p[3], e = 0.0f, c = 0.0f;
+        split(X, h, m);
 #pragma unroll
         for (int k = 0; k < D; k++) {
             // o is a small whole number of edges
             const float n = __fsub_rn(__fmaf_rn(o[k], inv_edge[k], 12582912.0f), 12582912.0f);
-            d[k] = __fmaf_rn(n, edge_hi[k], __fsub_rn(hi[k], h[k]));   // exact
-            dl[k] = __fmaf_rn(n, edge_lo[k], __fsub_rn(lo[k], l[k]));
-            p[k] = __fmul_rn(d[k], d[k]);
-            e = __fadd_rn(e, __fmaf_rn(d[k], d[k], -p[k]));
-            c = __fmaf_rn(d[k], dl[k], c);
+            const float u = __fmaf_rn(n, edge_hi[k], __fsub_rn(hi[k], h[k]));    // exact
+            const float v = __fmaf_rn(n, edge_mid[k], __fsub_rn(mid[k], m[k]));  // exact
+            const float w = __fmaf_rn(n, edge_lo[k], __fsub_rn(lo[k], l[k]));
+            const float d = __fadd_rn(u, v);
+            const float dl = __fadd_rn(__fsub_rn(v, __fsub_rn(d, u)), w);   // |u| >= |v|, or u = 0
+            p[k] = __fmul_rn(d, d);
+            e = __fadd_rn(e, __fmaf_rn(d, d, -p[k]));
+            c = __fmaf_rn(d, dl, c);
         }
         ff r2 = ff_two_sum(p[0], p[1]);
         r2.lo = __fadd_rn(r2.lo, e);
@@ -208,10 +220,10 @@ struct WendlandPairs {
         const float u = __fsub_rn(1.0f, s), ul = __fsub_rn(__fsub_rn(__fsub_rn(1.0f, u), s), ds);
         const float v = __fmaf_rn(4.0f, s, 1.0f);
         const float vl = __fmaf_rn(4.0f, ds, __fmaf_rn(4.0f, s, __fsub_rn(1.0f, v)));
-        const float u2 = __fmul_rn(u, u), u2l = __fmaf_rn(2.0f * u, ul, __fmaf_rn(u, u, -u2));
-        const float u4 = __fmul_rn(u2, u2), u4l = __fmaf_rn(2.0f * u2, u2l, __fmaf_rn(u2, u2, -u4));
+        const float u2 = __fmul_rn(u, u), u2l = __fmaf_rn(__fmaf_rn(2.0f, u, ul), ul, __fmaf_rn(u, u, -u2));
+        const float u4 = __fmul_rn(u2, u2), u4l = __fmaf_rn(__fmaf_rn(2.0f, u2, u2l), u2l, __fmaf_rn(u2, u2, -u4));
         const float w = __fmul_rn(u4, v);
-        const float wl = __fmaf_rn(u4l, v, __fmaf_rn(u4, vl, __fmaf_rn(u4, v, -w)));
+        const float wl = __fmaf_rn(u4l, vl, __fmaf_rn(u4l, v, __fmaf_rn(u4, vl, __fmaf_rn(u4, v, -w))));
         const ff q = ff_two_sum(sum.hi, w);
         sum.hi = q.hi;
         sum.lo = __fadd_rn(sum.lo, __fadd_rn(q.lo, wl));
