@@ -38,10 +38,10 @@
  *   - All work is issued on the stream given to sphfsi_create; getters and
  *     sphfsi_sync wait for it.  A getter that waits also comes after what is
  *     queued on the legacy default stream when it writes to device or pinned
- *     memory.  The state getters stage rows in device memory: 1 MB that a
- *     context always holds, and from the first larger read on a buffer of that
- *     read's size, at most 64 MB, kept until sphfsi_destroy (a read for which
- *     there is no more device memory makes do with the 1 MB).
+ *     memory.  The state getters stage rows in device memory: small reads in
+ *     the step's own scratch, larger ones in a buffer of the read's size, at
+ *     most 64 MB, kept until sphfsi_destroy (a read that cannot have it makes do
+ *     with the scratch).
  *   - A context is used by one host thread at a time.
  */
 #ifndef SPHFSI_H

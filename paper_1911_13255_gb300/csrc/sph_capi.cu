@@ -115,6 +115,8 @@ struct InstHost {
 
 }  // namespace
 
+constexpr size_t kReadLeast = (size_t)64 << 10;   // bytes of Fluid::bnd at least: it also stages state reads
+
 struct sphfsi_ctx {
     cudaStream_t st = nullptr;
     int dim = 2;
@@ -161,9 +163,7 @@ struct sphfsi_ctx {
     // row (original order), and the gathered rows
     int *d_orow = nullptr;
     double *d_spos = nullptr;
-    // staging of the state reads: kOneCopy bytes, and a larger buffer from the
-    // first larger read on
-    uint8_t *d_read0 = nullptr;
+    // staging of the state reads, from the first one that needs it
     void *d_read = nullptr;
     size_t read_bytes = 0;
     std::vector<uint8_t> h_read;   // at most kOneCopy bytes
@@ -707,6 +707,7 @@ struct Output {
     void *dst;      // caller's pointer (host or device), null: not asked for
     size_t row;     // bytes per row
     void *dev;      // its staged rows on the device
+    bool pageable = false;
 };
 
 // Pages of a fresh host array are mapped at their first touch: 3 us each from
@@ -726,12 +727,6 @@ cudaMemoryType memory_kind(const void *p)
     }
     return at.type;
 }
-bool pageable(const void *p) { return memory_kind(p) == cudaMemoryTypeUnregistered; }
-bool plain_host(const void *p)
-{
-    const cudaMemoryType t = memory_kind(p);
-    return t == cudaMemoryTypeUnregistered || t == cudaMemoryTypeHost;
-}
 
 // Work that the caller has queued on the default stream may still write or read
 // an output in memory that the device reaches: the context's stream, which
@@ -748,7 +743,7 @@ void touch_pages(const std::vector<Output> &outs, size_t n)
     const long os = sysconf(_SC_PAGESIZE);
     const size_t page = os > 0 ? (size_t)os : 4096, threads_from = (size_t)16 << 20;
     for (const Output &o : outs) {
-        if (!o.dst || !pageable(o.dst)) continue;
+        if (!o.dst || !o.pageable) continue;
         volatile char *p = (volatile char *)o.dst;
         const size_t bytes = n * o.row;
         const int64_t pages = (int64_t)((bytes + page - 1) / page);
@@ -758,11 +753,11 @@ void touch_pages(const std::vector<Output> &outs, size_t n)
     }
 }
 
-// Staging of the rows on the device: up to kOneCopy bytes in a buffer that
-// every context has from the start, more in one that grows with the first
-// larger read and stays, up to kReadMost bytes; a state beyond that, or one
-// whose larger buffer the device has no memory for, goes out in ranges of
-// rows (one pass over the slots each, 10 us on 3.0M particles).
+// Staging of the rows on the device: in Fluid::bnd, which carries nothing from
+// one step to the next, when they fit there; else in a buffer that the first
+// such read makes and that stays, of up to kReadMost bytes.  A state beyond
+// that, or one whose buffer the device has no memory for (it goes through bnd
+// then), goes out in ranges of rows, one pass over the slots each.
 constexpr size_t kOneCopy = (size_t)1 << 20, kReadMost = (size_t)64 << 20;
 
 // fill(outs, row0, rows) enqueues the kernel that writes rows [row0, row0 +
@@ -778,9 +773,9 @@ int read_rows(sphfsi_ctx *c, int n, std::vector<Output> outs, Fill &&fill)
     };
     const size_t total = staged((size_t)n);
     if (total == 0) return cuda_rc(cudaStreamSynchronize(c->st));
-    uint8_t *buf = (uint8_t *)c->d_read0;
-    size_t size = kOneCopy;
-    if (total > kOneCopy) {
+    uint8_t *buf = (uint8_t *)c->F.bnd;
+    size_t size = std::max((size_t)c->F.n * sizeof(float), kReadLeast);
+    if (total > size) {
         const size_t want = std::min(total, kReadMost);
         if (c->read_bytes < want) {
             if (c->d_read) {
@@ -802,10 +797,12 @@ int read_rows(sphfsi_ctx *c, int n, std::vector<Output> outs, Fill &&fill)
         }
     }
     bool one_copy = total <= kOneCopy, shared = false;
-    for (const Output &o : outs)
+    for (Output &o : outs)
         if (o.dst) {
-            one_copy = one_copy && plain_host(o.dst);
-            shared = shared || !pageable(o.dst);
+            const cudaMemoryType kind = memory_kind(o.dst);
+            o.pageable = kind == cudaMemoryTypeUnregistered;
+            one_copy = one_copy && (o.pageable || kind == cudaMemoryTypeHost);
+            shared = shared || !o.pageable;
         }
     if (shared) TRY(after_default_stream(c));
     if (!one_copy) touch_pages(outs, (size_t)n);
@@ -1252,7 +1249,6 @@ int sphfsi_finalize(sphfsi_ctx *c)
     }
     TRY(dalloc(c, &F.bsum, 4096));
     TRY(dalloc(c, &F.gbar, 2));
-    TRY(dscratch(c, &c->d_read0, kOneCopy));
     // neighbour rows (tuned): about 20 (2-D) or 80 (3-D) neighbours per fluid
     // particle on a lattice, wall neighbours included.  On from 32 768 fluid
     // particles in 2-D (2 lanes per target) and 16 384 in 3-D (4).  Step with the
@@ -1277,11 +1273,13 @@ int sphfsi_finalize(sphfsi_ctx *c)
         with_rows += form[b];
     }
     F.only = -1;
-    int *d_form = nullptr;
-    TRY(dscratch(c, &d_form, B));
-    TRY(upload(c, d_form, form));
-    F.form = d_form;
     c->two_forms = with_rows > 0 && with_rows < B;
+    if (c->two_forms) {
+        int *d_form = nullptr;
+        TRY(dscratch(c, &d_form, B));
+        TRY(upload(c, d_form, form));
+        F.form = d_form;
+    }
     if (with_rows) {
         F.list = 1;
         F.lanes = D == 3 ? 4 : 2;
@@ -1303,7 +1301,7 @@ int sphfsi_finalize(sphfsi_ctx *c)
     TRY(dalloc(c, &F.nbc, nf));
     for (int p = 0; p < 2; p++) TRY(dscratch(c, &F.part[p], nf));
     TRY(dscratch(c, &F.part_n, 2));
-    TRY(dscratch(c, &F.bnd, nf));
+    TRY(dscratch(c, &F.bnd, std::max<size_t>((size_t)nf, kReadLeast / sizeof(float))));
     // held pair configuration: off (rebuilt every step); the first step builds it
     F.held_n = 1;
     TRY(dalloc(c, &F.held, 3));
@@ -1737,7 +1735,7 @@ int sphfsi_get_solid_positions_async(sphfsi_ctx *c, double *r)
 int sphfsi_get_solid_positions_all(sphfsi_ctx *c, double *r)
 {
     TRY(check_ctx(c, true));
-    if (r && !pageable(r)) TRY(after_default_stream(c));
+    if (r && memory_kind(r) != cudaMemoryTypeUnregistered) TRY(after_default_stream(c));
     TRY(sphfsi_get_solid_positions_async(c, r));
     return cuda_rc(cudaStreamSynchronize(c->st));
 }
