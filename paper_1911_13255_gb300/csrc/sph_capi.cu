@@ -146,12 +146,14 @@ struct sphfsi_ctx {
     // per-stage CUDA events (sphfsi_set_profiling), by index: 0 start, 2
     // binning, 1 neighbour rows, 3 reinit, 5 momentum, 6 continuity (main
     // stream); 4 branch start, 7 coupling force done, 8 sub-steps done (side
-    // stream); 9 end of step
+    // stream); 9 end of step; 10 and 11 around the rows where they are built
+    // behind the fork (late_rows)
     static constexpr int kStages = 8;
-    static constexpr int kEvents = 10;
+    static constexpr int kEvents = 12;
     bool profiling = false;
     cudaEvent_t ev[kEvents] = {};
     int kernels_per_step = 0;
+    bool late_rows = false;    // the last step's rows were built behind the fork
     bool fork_first = false;   // the solid branch starts before the neighbour rows are built
     bool two_forms = false;    // some instances take rows, some the cell form (until the tuning is set)
     int max_reach = 1;   // largest cell reach of the instances (sphfsi_params::cell_reach)
@@ -329,7 +331,7 @@ int enqueue_step(sphfsi_ctx *c, double dt)
     // density reinitialisation (no-op on other steps).  Where the solid branch
     // is the longer one (fork_first) the rows wait until it has started: the
     // reinitialisation, which it waits for, then visits the cells.
-    const bool late_rows = c->F.list && c->fork_first && c->S.n;
+    const bool late_rows = c->late_rows = c->F.list && c->fork_first && c->S.n;
     Fluid rows = c->F, cells = c->F;
     if (late_rows || c->two_forms) cell_form(c, cells);
     if (c->two_forms) rows.only = 1, cells.only = 0;
@@ -360,7 +362,11 @@ int enqueue_step(sphfsi_ctx *c, double dt)
         TRY(mark(c, 8, c->side));
         TRY(cuda_rc(cudaEventRecord(c->join_ev, c->side)));
     }
-    if (late_rows) TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
+    if (late_rows) {
+        TRY(mark(c, 10));
+        TRY(launch_pairlist(c->bt, c->F, c->W, c->S, D, st));
+        TRY(mark(c, 11));
+    }
     TRY(pair_loop(launch_momentum));
     TRY(mark(c, 5));
     TRY(pair_loop(launch_density));
@@ -2445,11 +2451,11 @@ int sphfsi_stage_times(sphfsi_ctx *c, float *ms, int n)
     auto el = [&](int a, int b, float *o) { return cuda_rc(cudaEventElapsedTime(o, c->ev[a], c->ev[b])); };
     // events: 0 start, 2 binning, 3 reinit, 5 momentum, 6 continuity (main
     // stream); 4 branch start, 7 coupling force done, 8 sub-steps done (side
-    // stream); 9 end of step
+    // stream); 9 end of step; 10, 11 around rows behind the fork
     TRY(el(0, 2, &ms[0]));
-    TRY(el(2, 1, &ms[7]));
+    TRY(c->late_rows ? el(10, 11, &ms[7]) : el(2, 1, &ms[7]));
     TRY(el(1, 3, &ms[1]));
-    TRY(el(3, 5, &ms[2]));
+    TRY(el(c->late_rows ? 11 : 3, 5, &ms[2]));
     TRY(el(5, 6, &ms[4]));
     if (c->S.n) {
         float fin_a = 0.f, fin_b = 0.f;
