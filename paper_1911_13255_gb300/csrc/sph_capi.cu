@@ -618,42 +618,47 @@ int solid_windows(sphfsi_ctx *c, const std::vector<int> &ptr, const std::vector<
     Solid &S = c->S;
     S.win_ctas = 0;
     if (c->B != 1 || S.n == 0) return SPHFSI_OK;
-    int dev = 0, nsm = 0, own = 0, threads = 0;
+    int dev = 0, nsm = 0, own = 0, least = 0;
     TRY(cuda_rc(cudaGetDevice(&dev)));
     TRY(cuda_rc(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)));
     // the sub-steps' share of 80 % of momentum and continuity (about 20 us and
     // 0.9 ns per fluid particle in 3-D, 0.6 ns in 2-D)
     const double loops = 20.0 + (c->dim == 3 ? 0.9e-3 : 0.6e-3) * (double)c->F.n;
-    solid_window_shape(c->dim, S.n, nsm, 0.8 * loops / std::max(1.0, first_substeps(c->ih[0])), &own, &threads);
-    const int ctas = (S.n + own - 1) / own;
-    std::vector<int4> win(ctas);
-    std::vector<int2> wait(ctas);
+    solid_window_shape(c->dim, S.n, nsm, 0.8 * loops / std::max(1.0, first_substeps(c->ih[0])), &own, &least);
+    std::vector<int4> win;
     int slots = 0;
-    for (int k = 0; k < ctas; k++) {
-        const int a0 = k * own, a1 = std::min(a0 + own, S.n);
-        int lo = a0, hi = a1;
-        for (int a = a0; a < a1; a++)
-            if (ptr[a + 1] > ptr[a]) {
-                lo = std::min(lo, nbi[ptr[a]]);
-                hi = std::max(hi, nbi[ptr[a + 1] - 1] + 1);
-            }
-        win[k] = make_int4(a0, a1 - a0, lo, hi - lo);
-        wait[k] = make_int2(lo / own, (hi - 1) / own);
-        slots = std::max(slots, hi - lo);
+    for (;; own = std::max(least, own / 2)) {   // fewer particles have smaller windows
+        win.resize((S.n + own - 1) / own);
+        slots = 0;
+        for (int k = 0; k < (int)win.size(); k++) {
+            const int a0 = k * own, a1 = std::min(a0 + own, S.n);
+            int lo = a0, hi = a1;
+            for (int a = a0; a < a1; a++)
+                if (ptr[a + 1] > ptr[a]) {
+                    lo = std::min(lo, nbi[ptr[a]]);
+                    hi = std::max(hi, nbi[ptr[a + 1] - 1] + 1);
+                }
+            win[k] = make_int4(a0, a1 - a0, lo, hi - lo);
+            slots = std::max(slots, hi - lo);
+        }
+        if (solid_window_fits(c->dim, (int)win.size(), solid_window_threads(c->dim, own), slots, own)) break;
+        if (own <= least) return SPHFSI_OK;
     }
+    const int ctas = (int)win.size();
+    std::vector<int2> wait(ctas);
+    for (int k = 0; k < ctas; k++) wait[k] = make_int2(win[k].z / own, (win[k].z + win[k].w - 1) / own);
     for (int k = 0; k < ctas; k++)   // both directions
         for (int j = win[k].z / own; j <= (win[k].z + win[k].w - 1) / own; j++) {
             wait[j].x = std::min(wait[j].x, k);
             wait[j].y = std::max(wait[j].y, k);
         }
-    if (!solid_window_fits(c->dim, ctas, threads, slots, own)) return SPHFSI_OK;
     TRY(dscratch(c, &S.win, ctas));
     TRY(dscratch(c, &S.win_wait, ctas));
     TRY(dscratch(c, &S.win_flag, 32 * (size_t)ctas));
     TRY(upload(c, S.win, win));
     TRY(upload(c, S.win_wait, wait));
     S.win_ctas = ctas;
-    S.win_threads = threads;
+    S.win_threads = solid_window_threads(c->dim, own);
     S.win_slots = slots;
     S.win_own = own;
     return SPHFSI_OK;

@@ -505,9 +505,11 @@ int launch_debug_pairs(const Batch &bt, const Fluid &f, const Walls &w, const So
 int launch_solid_setup_fill(const Batch &bt, Solid &s, const int *nbi, int dim, cudaStream_t st);
 // P0: host copy of instance 0's constants (used when the batch holds one instance)
 int launch_solid_substeps(const Batch &bt, Solid &s, const Phys &P0, int dim, int *path, cudaStream_t st);
-// plan of the windowed sub-step kernel: particles and threads per CTA, and
-// whether the device can hold the grid with these windows (sph_solid.cu)
-void solid_window_shape(int dim, int n, int nsm, double sub_us, int *own, int *threads);
+// plan of the windowed sub-step kernel: particles per CTA and their lower
+// bound, threads per CTA, and whether the device can hold the grid with these
+// windows (sph_solid.cu)
+void solid_window_shape(int dim, int n, int nsm, double sub_us, int *own, int *least);
+int solid_window_threads(int dim, int own);
 int solid_window_fits(int dim, int ctas, int threads, int slots, int own);
 // learned sub-stepper: features into x (n x 64), then, from the network's
 // outputs (n x 16), candidate, residual and accept / reject (sph_solid.cu)

@@ -1878,9 +1878,10 @@ static size_t window_smem(int dim, int slots, int own)
     return (size_t)slots * 16 * (dim == 3 ? 4 : 2) + (size_t)own * dim * dim * sizeof(float);
 }
 
-// Shape of the windowed kernel for a body of n particles: particles per CTA
-// and threads per CTA.  At most one CTA per SM, and at least 32 particles each,
-// since a CTA's phase costs a few L2 round trips however little it holds.
+// Shape of the windowed kernel for a body of n particles: particles per CTA,
+// and the least that it may be.  At most one CTA per SM, and at least 32
+// particles each, since a CTA's phase costs a few L2 round trips however little
+// it holds.
 // Between these bounds, as many particles per CTA as let a sub-step take about
 // sub_us: a CTA's 512 threads of 128 registers leave its SM to nothing else, so
 // when the fluid loops are the longer branch the sub-steps should hide behind
@@ -1888,18 +1889,18 @@ static size_t window_smem(int dim, int slots, int own)
 // 2-D (P particles per CTA).  3-D duct, 375k fluid and 8160 solid particles: step
 // 881 us with 152 CTAs, 806 with 76, 775 with 38, 820 with 24; 2-D gate of 6400
 // particles, the longer branch there: 188 us with 152, 186 with 100, 278 with 25.
-void solid_window_shape(int dim, int n, int nsm, double sub_us, int *own, int *threads)
+void solid_window_shape(int dim, int n, int nsm, double sub_us, int *own, int *least)
+{
+    *least = std::max(32, (n + nsm - 1) / nsm);
+    const double fit = dim == 3 ? (sub_us - 8.0) / 0.055 : (sub_us - 4.0) / 0.02;
+    const int P = (int)std::min(std::max(fit, (double)*least), (double)kWinThreads);
+    *own = std::max(std::min(P, n), *least);
+}
+
+int solid_window_threads(int dim, int own)
 {
     const int L = dim == 3 ? kWinL<3> : kWinL<2>;
-    const int least = std::max(32, (n + nsm - 1) / nsm);
-    const double fit = dim == 3 ? (sub_us - 8.0) / 0.055 : (sub_us - 4.0) / 0.02;
-    int P = (int)std::min(std::max(fit, (double)least), (double)kWinThreads);
-    P = std::max(std::min(P, n), least);
-    int T = (P * L + 31) / 32 * 32;
-    if (T > kWinThreads) T = kWinThreads;
-    if (T < (P + 31) / 32 * 32) T = (P + 31) / 32 * 32;
-    *own = P;
-    *threads = T;
+    return std::max(std::min((own * L + 31) / 32 * 32, kWinThreads), (own + 31) / 32 * 32);
 }
 
 // Can the device hold the plan's grid at once?  (0: no)
