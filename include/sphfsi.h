@@ -412,8 +412,10 @@ typedef struct {
                               a row (at most 64 in 2-D, 128 in 3-D; a fuller row falls back to the
                               cell visit for that particle), and stream the rows in momentum,
                               continuity and reinitialisation; not with tiles or cell_reach 2
-                              (default 1 from 16 384 fluid particles in the context in 3-D and
-                              32 768 in 2-D, else 0) */
+                              (default 1 from 16 384 fluid particles in 3-D and 32 768 in 2-D,
+                              else 0: by instance, in contexts of 262 144 particles and more by
+                              the total.  A batch with both kinds steps each instance in its own
+                              form and reads 1 here; sphfsi_set_tuning gives all one form) */
     int32_t list_lanes;    /* 1, 8, 16 or 32 (default 1; 0 keeps the current value): kept for
                               callers that set it; one row build, a warp per cell, serves them all */
 } sphfsi_tuning;

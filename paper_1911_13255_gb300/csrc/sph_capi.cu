@@ -1263,11 +1263,13 @@ int sphfsi_finalize(sphfsi_ctx *c)
     // neighbour rows (tuned): about 20 (2-D) or 80 (3-D) neighbours per fluid
     // particle on a lattice, wall neighbours included.  On from 32 768 fluid
     // particles in 2-D (2 lanes per target) and 16 384 in 3-D (4).  Step with the
-    // cell form and with rows: 2-D channels of 33k particles 87 against 71 us,
-    // batches of 171k and 577k 248 and 574 against 234 and 485; 3-D tanks of 4k,
-    // 11k, 24k and 62k 219, 151, 202 and 393 against 218, 151, 182 and 320.
-    // Smaller problems gain little or nothing (2-D channel of 10k 65 -> 60 us, dam
-    // break of 14k 90 -> 87; 3-D as above).
+    // cell form and with rows: 2-D channels of 10k and 33k particles 65 and 87
+    // against 60 and 71 us, a dam break of 14k 90 against 87, batches of 171k and
+    // 577k 248 and 574 against 234 and 485; 3-D tanks of 4k, 11k, 24k and 62k 219,
+    // 151, 202 and 393 against 218, 151, 182 and 320.  So in 3-D the line lies
+    // between the sizes that gain nothing and those that do; in 2-D rows would pay
+    // from some 8k, and smaller problems keep the form (and the order of sums) that
+    // they have always had by default, for a difference of 3 to 8 %.
     // The form decides the order of a particle's sums, and a batch equals its
     // instances stepped alone to the last bit: an instance of a batch takes the
     // form that it takes alone.  (Contexts of 262 144 particles and more, whose

@@ -235,6 +235,8 @@ struct ShapeSums {
     ff f, w, s;
 };
 
+// (each lane's own sum is such a pair: the few additions here add 2^-48 of the
+// sum each, as every pair's did)
 template <int L>
 __device__ __forceinline__ ff group_sum_ff(ff v)
 {

@@ -736,13 +736,6 @@ __device__ __forceinline__ float group_sum(float v)
     for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-template <int L>
-__device__ __forceinline__ double group_sum_d(double v)
-{
-#pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // p_i - p_j of Eq. eqeos without cancellation: with a = 1 + drho_i / rho0 and
 // b = 1 + drho_j / rho0, p_i - p_j = (rho0 c^2 / 7) (a^7 - b^7)
