@@ -387,11 +387,22 @@ int request_rebuild(sphfsi_ctx *c)
     return cuda_rc(cudaMemsetAsync(c->F.held, 0xff, sizeof(int), c->st));
 }
 
+// The rows of the pair configuration that is held now: its records keep the
+// positions of its build, and its cell starts stay.
+int rows_of_held(sphfsi_ctx *c)
+{
+    Fluid F = c->F;
+    F.held_n = 1;   // the row build skips steps that do not rebuild
+    if (c->two_forms) F.only = 1;
+    TRY(cuda_rc(cudaMemsetAsync(F.part_n, 0, 2 * sizeof(int), c->st)));
+    return launch_pairlist(c->bt, F, c->W, c->S, c->dim, c->st);
+}
+
 // After the device state has been replaced, what lives beside it: equal phase
 // counts for the CTAs of the windowed sub-step kernel (a time-out leaves them
 // unequal); the lists that follow from the rows' words; and with a held
-// configuration, a rebuild at the next step if this context streams rows and
-// the state, which came from one that did not, has none.
+// configuration, the rows if this context streams them and the state, which
+// came from one that did not, has none.
 int scratch_from_state(sphfsi_ctx *c)
 {
     if (c->S.win_ctas)
@@ -402,7 +413,7 @@ int scratch_from_state(sphfsi_ctx *c)
     uint32_t word = 0;
     TRY(cuda_rc(cudaMemcpyAsync(&word, c->F.nbc, sizeof(word), cudaMemcpyDeviceToHost, c->st)));
     TRY(cuda_rc(cudaStreamSynchronize(c->st)));
-    return word ? SPHFSI_OK : request_rebuild(c);
+    return word ? SPHFSI_OK : rows_of_held(c);
 }
 
 int check_ctx(sphfsi_ctx *c, bool need_final)
@@ -2143,8 +2154,9 @@ int sphfsi_set_tuning(sphfsi_ctx *c, const sphfsi_tuning *t)
     c->F.rows = t->rows;
     c->two_forms = false;   // one shape for all
     // a held configuration built without rows has none to stream
-    if (t->list && !c->F.list && held_on(c->F)) TRY(request_rebuild(c));
+    const bool no_rows = t->list && !c->F.list && held_on(c->F);
     c->F.list = t->list;
+    if (no_rows) TRY(rows_of_held(c));
     if (t->list_lanes) c->F.list_lanes = t->list_lanes;
     c->S.force_lane_path = t->solid_variant;
     if (c->gexec) {
