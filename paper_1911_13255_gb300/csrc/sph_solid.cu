@@ -370,6 +370,7 @@ __global__ void __launch_bounds__(kSolidBlock) k_solid_substeps(Batch bt, Solid 
 constexpr int kCThreads = 512;
 constexpr int kLanes = 4;
 constexpr int kPPC = kCThreads / kLanes;
+constexpr int kOwnFloats = 21;   // floats of a particle in shared memory beside its stress and velocity
 constexpr int kClusterMax = 16;
 static_assert(kClusterMax * kPPC == kClusterBody && kClusterMax * kSolidCta == kClusterBody, "one cluster's body");
 
@@ -451,9 +452,15 @@ __device__ __forceinline__ float square3(float x, float y, float z)
 // K sub-steps of one instance's body (slots [s0, s0 + ns)) by one cluster
 template <int D>
 __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, Ctl *ctl, int s0, int ns, float4 *sQ,
-                                                 float4 *sV, unsigned rank)
+                                                 float4 *sV, float *sOwn, unsigned rank)
 {
     const int g = threadIdx.x / kLanes, lane = threadIdx.x % kLanes;
+    // of the group's first lane: B0, and in 3-D the rests of H and v (add_rest).
+    // In shared memory, as every register counts: the cluster's CTAs have to fit
+    // beside a block of the fluid loops that run meanwhile (104 registers a
+    // thread leave room for one of 128 threads; with 124, all of it in registers,
+    // an 11-CTA body waited 10 us for empty SMs: stage 29 -> 39 us)
+    float *const B = sOwn + kOwnFloats * g, *const Hr = B + 9, *const vr = B + 18;
     const int la = (int)rank * kPPC + g;
     const int a = s0 + la;
     const bool own = la < ns;
@@ -463,9 +470,8 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
     const float dts = (float)dtsd, hdts = 0.5f * dts;
     const float inv_rhoS = 1.0f / P.rhoS, inv_mS = 1.0f / P.mS;
 
-    float H[9], B[9], fF[3] = {0.f, 0.f, 0.f};
-    float Hr[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, vr[3] = {0.f, 0.f, 0.f};   // 3-D: rests of H and v (add_rest)
-    double x = 0, y = 0, z = 0, xs = 0, ys = 0, zs = 0, as[3] = {0, 0, 0};
+    float H[9], fF[3] = {0.f, 0.f, 0.f};
+    double x = 0, y = 0, z = 0, as[3] = {0, 0, 0};
     bool cons = true;
     float vmax = 0.0f, amax = 0.0f;
     int q0 = 0, q1 = 0;
@@ -476,11 +482,15 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
             for (int i = 0; i < D * D; i++) {
                 H[i] = s.H[9 * a + i];
                 B[i] = s.B0[9 * a + i];
+                Hr[i] = 0.0f;
             }
-            for (int k = 0; k < D; k++) fF[k] = s.fF[3 * a + k];
-            x = xs = s.x[a];
-            y = ys = s.y[a];
-            if (D == 3) z = zs = s.z[a];
+            for (int k = 0; k < D; k++) {
+                fF[k] = s.fF[3 * a + k];
+                vr[k] = 0.0f;
+            }
+            x = s.x[a];
+            y = s.y[a];
+            if (D == 3) z = s.z[a];
             cons = s.cons[a] != 0;
             sV[g] = s.v4[a];
         }
@@ -519,6 +529,7 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
             }
         }
         for (int i = 0; i < D * D; i++) M[i] = D == 3 ? strand_sum(M[i], M2[i]) : group_sum(M[i]);
+        if (lane != 0) return;
         for (int i = 0; i < D; i++)
             for (int j = 0; j < D; j++) {
                 float v = 0.0f;
@@ -658,14 +669,14 @@ __device__ __forceinline__ void solid_lanes_body(const Solid &s, const Phys &P, 
     if (own && lane == 0) {
         for (int i = 0; i < D * D; i++) s.H[9 * a + i] = H[i];
         s.v4[a] = sV[g];
+        const double idt = 1.0 / dt;   // (the start positions are still in place)
+        s.vbar[3 * a] = (x - s.x[a]) * idt;
+        s.vbar[3 * a + 1] = (y - s.y[a]) * idt;
+        s.vbar[3 * a + 2] = D == 3 ? (z - s.z[a]) * idt : 0.0;
+        for (int k = 0; k < 3; k++) s.abar[3 * a + k] = as[k] * idt;
         s.x[a] = x;
         s.y[a] = y;
         if (D == 3) s.z[a] = z;
-        const double idt = 1.0 / dt;
-        s.vbar[3 * a] = (x - xs) * idt;
-        s.vbar[3 * a + 1] = (y - ys) * idt;
-        s.vbar[3 * a + 2] = D == 3 ? (z - zs) * idt : 0.0;
-        for (int k = 0; k < 3; k++) s.abar[3 * a + k] = as[k] * idt;
     }
     float vm = warp_max(vmax), am = warp_max(amax);
     if ((threadIdx.x & 31) == 0 && own) {
@@ -697,13 +708,14 @@ __global__ void __launch_bounds__(kCThreads) k_solid_cluster(Batch bt, Solid s)
     constexpr int QR = D == 3 ? 3 : 1;   // float4 rows of Q per particle
     __shared__ float4 sQ[kPPC * QR];
     __shared__ float4 sV[kPPC];
+    __shared__ float sOwn[kPPC * kOwnFloats];
     __shared__ int s_inst;
     const unsigned rank = cluster_rank();
     for (;;) {
         const int b = next_instance(s.queue, &s_inst, rank);
         if (b >= bt.B) break;
         const Inst &In = bt.I[b];
-        solid_lanes_body<D>(s, In.P, bt.ctl + b, In.s0, In.ns, sQ, sV, rank);
+        solid_lanes_body<D>(s, In.P, bt.ctl + b, In.s0, In.ns, sQ, sV, sOwn, rank);
     }
 }
 
@@ -715,7 +727,8 @@ __global__ void __launch_bounds__(kCThreads) k_solid_cluster_one(Solid s, const 
     constexpr int QR = D == 3 ? 3 : 1;
     __shared__ float4 sQ[kPPC * QR];
     __shared__ float4 sV[kPPC];
-    solid_lanes_body<D>(s, P, ctl, 0, s.n, sQ, sV, cluster_rank());
+    __shared__ float sOwn[kPPC * kOwnFloats];
+    solid_lanes_body<D>(s, P, ctl, 0, s.n, sQ, sV, sOwn, cluster_rank());
 }
 
 // ---------------------------------------------------------------------------
