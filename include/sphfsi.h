@@ -335,9 +335,13 @@ int sphfsi_debug_neighbors(sphfsi_ctx *c, int which, int64_t *ptr, int64_t *idx,
  * when the body fits one thread-block cluster of at most 16 CTAs x 128
  * particles and the device can launch it -- in 2-D with at most 24 static
  * neighbours per particle the one-thread-per-particle variant, otherwise the
- * four-lanes-per-particle variant -- else the cooperative grid kernel);
- * 1 the four-lane cluster variant where it fits; 2 always the cooperative
+ * four-lanes-per-particle variant -- else a cooperative grid kernel, which a
+ * single 3-D body above 512 particles takes as well, with the same bits);
+ * 1 the four-lane cluster variant where it fits; 2 always a cooperative
  * grid kernel (single-instance contexts only; SPHFSI_E_INVAL in a batch).
+ * The grid kernel's CTAs exchange particles with their neighbours only,
+ * through shared-memory windows; where those do not fit, it has a barrier of
+ * all CTAs per phase.
  * All compute the same sub-steps (Section 3.3); the choice exists to test
  * and compare them.  In a batch the cluster kernels are persistent: as many
  * clusters as fit on the device take instances from a device queue. */

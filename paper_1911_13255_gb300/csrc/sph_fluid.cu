@@ -139,7 +139,7 @@ __device__ __forceinline__ void momentum_one(const Batch &bt, const Fluid &f, co
 // events, all targets alike -> in three kinds): 375k particles 637 -> 384 us,
 // 3.0M particles 2.49 -> 1.97 ms; reinitialisation 179 -> 107 us and 847 -> 712 us
 // per step.  With four entries per load and the pairs of the reinitialisation in
-// FP32 these are now 245 us, 1.72 ms, 75 us and 448 us.
+// FP32 these are now 248 us, 1.76 ms, 81 us and 495 us.
 template <int D, int L, bool CP, bool TILE, int FORM>
 __global__ void __launch_bounds__(kMaxBlock, FORM == 1 ? 3 : 4) k_momentum(Batch bt, Fluid f, Walls w, Solid s)
 {
