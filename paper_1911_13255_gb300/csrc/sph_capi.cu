@@ -155,6 +155,7 @@ struct sphfsi_ctx {
     int kernels_per_step = 0;
     bool late_rows = false;    // the last step's rows were built behind the fork
     bool fork_first = false;   // the solid branch starts before the neighbour rows are built
+    std::vector<int> form;     // per instance: 1 if it takes rows by default
     bool two_forms = false;    // some instances take rows, some the cell form (until the tuning is set)
     int max_reach = 1;   // largest cell reach of the instances (sphfsi_params::cell_reach)
     // side stream for the solid branch, which runs beside momentum and continuity
@@ -402,7 +403,7 @@ int rows_of_held(sphfsi_ctx *c)
 // counts for the CTAs of the windowed sub-step kernel (a time-out leaves them
 // unequal); the lists that follow from the rows' words; and with a held
 // configuration, the rows if this context streams them and the state, which
-// came from one that did not, has none.
+// came from one that did not (or not for all of its instances), has none.
 int scratch_from_state(sphfsi_ctx *c)
 {
     if (c->S.win_ctas)
@@ -410,10 +411,13 @@ int scratch_from_state(sphfsi_ctx *c)
     if (c->F.n == 0) return SPHFSI_OK;
     TRY(launch_row_parts(c->F, c->st));
     if (!c->F.list || !held_on(c->F)) return SPHFSI_OK;
-    uint32_t word = 0;
-    TRY(cuda_rc(cudaMemcpyAsync(&word, c->F.nbc, sizeof(word), cudaMemcpyDeviceToHost, c->st)));
+    std::vector<uint32_t> first(c->B, 1u);   // each instance's first word
+    for (int b = 0; b < c->B; b++)
+        if (c->ih[b].nf > 0 && (!c->two_forms || c->form[b]))
+            TRY(cuda_rc(cudaMemcpyAsync(&first[b], c->F.nbc + c->ih[b].d.f0, sizeof(uint32_t), cudaMemcpyDeviceToHost,
+                                        c->st)));
     TRY(cuda_rc(cudaStreamSynchronize(c->st)));
-    return word ? SPHFSI_OK : rows_of_held(c);
+    return std::count(first.begin(), first.end(), 0u) ? rows_of_held(c) : SPHFSI_OK;
 }
 
 int check_ctx(sphfsi_ctx *c, bool need_final)
@@ -1289,7 +1293,8 @@ int sphfsi_finalize(sphfsi_ctx *c)
     F.n = (int)nf;
     c->S.n = (int)ns;
     cell_form(c, F);
-    std::vector<int> form(B, 0);
+    std::vector<int> &form = c->form;
+    form.assign(B, 0);
     int with_rows = 0;
     for (int b = 0; b < B; b++) {
         const int64_t size = small ? c->ih[b].nf : nf;
@@ -2152,10 +2157,10 @@ int sphfsi_set_tuning(sphfsi_ctx *c, const sphfsi_tuning *t)
     c->F.split_records = t->records == 1 ? 1 : 0;
     c->F.bin_fused = t->records == 2 ? 1 : 0;
     c->F.rows = t->rows;
-    c->two_forms = false;   // one shape for all
     // a held configuration built without rows has none to stream
-    const bool no_rows = t->list && !c->F.list && held_on(c->F);
+    const bool no_rows = t->list && (!c->F.list || c->two_forms) && held_on(c->F);
     c->F.list = t->list;
+    c->two_forms = false;   // one shape for all
     if (no_rows) TRY(rows_of_held(c));
     if (t->list_lanes) c->F.list_lanes = t->list_lanes;
     c->S.force_lane_path = t->solid_variant;
@@ -2209,6 +2214,7 @@ int sphfsi_autotune(sphfsi_ctx *c, double dt_F, int32_t steps, sphfsi_tuning *be
         }
         if (!save) {
             c->F.list = keep.list;   // the restored rows are the ones of the snapshot's form
+            c->two_forms = keep_two;
             TRY(scratch_from_state(c));
         }
         return cuda_rc(cudaStreamSynchronize(c->st));

@@ -231,8 +231,8 @@ struct Fluid {
 // nbc flags: solid particles in one of the target's neighbour cells (the pair
 // loops visit those cells for the solid candidates); the row overflowed (the
 // target takes the cell visit for everything); the word is a built row's (a
-// rebuild step without rows clears slot 0's word, so nbc[0] == 0 says that the
-// rows are not those of the current pair configuration)
+// rebuild step that builds no rows for an instance clears its first slot's word,
+// so 0 there says that its rows are not those of the current pair configuration)
 constexpr uint32_t kListSolid = 1u << 22, kListOver = 1u << 23, kListBuilt = 1u << 24;
 constexpr uint32_t kListCountMask = 0x7ffu;
 constexpr uint32_t kListWalls = kListCountMask << 11;   // nW != 0

@@ -344,11 +344,11 @@ __global__ void __launch_bounds__(32 * kRowWarps, D == 3 ? 5 : 8) k_pairlist_cel
     const int a0 = f.cstart[cell], a1 = f.cstart[cell + 1];
     if (a0 >= a1) return;
     RowWarp<D> &sw = s_warp[threadIdx.x >> 5];
+    const Inst &In = bt.I[f.inst[a0]];
     if (!takes(f, f.inst[a0])) {
-        if (a0 == 0 && lane == 0) f.nbc[0] = kListBuilt;   // (the other instances' rows are)
+        if (a0 == In.f0 && lane == 0) f.nbc[a0] = 0u;   // no rows of this configuration
         return;
     }
-    const Inst &In = bt.I[f.inst[a0]];
     const Grid &g = In.g;
     const float rc2 = In.P.rc2F, reach2 = rc2 * 1.0001f;   // the box test's rounding stays within the margin
     constexpr int NR = D == 3 ? 9 : 3;

@@ -334,13 +334,12 @@ __global__ void k_bin_all(Batch bt, Fluid f, Solid s, int step, double dt_fixed,
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) {
         *f.nlive = 0;
-        if (rebuild_step(bt, f)) {
-            f.part_n[0] = f.part_n[1] = 0;   // filled by the row build
-            if (!f.list) f.nbc[0] = 0u;      // the rows, if there are any, are an older configuration's
-        }
+        if (rebuild_step(bt, f)) f.part_n[0] = f.part_n[1] = 0;   // filled by the row build
         f.scan_ctl[0] = 0u;    // the scan's tickets
         f.scan_ctl[1] += 1u;   // and its epoch: this binning's tile states
     }
+    // without rows, those that there are are an older configuration's
+    if (!f.list && t < bt.B && bt.I[t].nf && rebuild_step(bt, f)) f.nbc[bt.I[t].f0] = 0u;
     // dt_F once for a block whose particles share an instance (FP64 divisions)
     __shared__ double s_dt;
     const int t0 = blockIdx.x * blockDim.x, t1 = t0 + (int)blockDim.x - 1;
@@ -897,10 +896,10 @@ __global__ void __launch_bounds__(kBinFusedThreads, 1)
     int *status = &bt.ctl[0].status;
     const int np = f.n + s.n;
     // (1) step control, drift, cell keys, histograms
-    if (gt == 0) {
-        *f.nlive = f.part_n[0] = f.part_n[1] = 0;
-        if (!f.list) f.nbc[0] = 0u;
-    }
+    if (gt == 0) *f.nlive = f.part_n[0] = f.part_n[1] = 0;
+    if (!f.list)
+        for (int b = gt; b < bt.B; b += gs)
+            if (bt.I[b].nf) f.nbc[bt.I[b].f0] = 0u;
     for (int t = gt; t < np + (step ? bt.B : 0); t += gs) bin_one<D>(bt, f, s, t, step, dt_fixed, K_fixed);
     if (!grid_barrier(f.gbar, status, bt.spin, bt.fail)) return;
     // (2) exclusive scan of [fluid counts | solid counts]
